@@ -196,8 +196,7 @@ sp_status sp_step(sp_ctx* ctx, int n_steps);
  * SP_F_ratio; the other fields are 0).  out: host [n_fields][ncells(inst)].
  * In reproducible runs (FP64, or sp_set_reproducible on) kind 0 sums each
  * cell in source order, so the fields are bit-identical from run to run;
- * it puts the cells' particles in that order on the device first, which is
- * the order the next step would restore anyway (no later result changes).
+ * the steps and uploads of such a run leave the particles in that order.
  * With an FP32 state, kind 0 forms the per-cell quotients as products of
  * reciprocals (a few ulps from the FP64 mode's quotients).  When out is
  * page-locked host memory mapped for the device (cudaHostAlloc,
@@ -329,7 +328,7 @@ sp_status sp_free(sp_ctx* ctx);
  *           r-th kept particle of cell c, in ascending index order
  *   stream  cudaStream_t or NULL; the call is asynchronous on it.
  * Scratch lives in a file-scope __device__ array sized for ncells <=
- * 1,048,576 (8 MiB, held by every GPU that loads the library until exit);
+ * 1,048,576 (4 MiB, held by every GPU that loads the library until exit);
  * larger ncells, or n > 2^30 keys, return SP_ERR_CAPACITY with a message.
  * Cells of up to 1024 entries are put in order by one warp each, larger
  * ones by a block each (a cell of 2^20 entries takes a few tenths of a

@@ -3,14 +3,15 @@
 // Per step the driver enqueues, on the context's stream:
 //   1. k_plan + k_collide (batches of cells per warp) and its
 //      big-cell launch (one warp per cell with a large staging area):
-//      gather through perm in stable order -> Step 3 moments -> Step 4
+//      gather through perm -> Step 3 moments -> Step 4
 //      DSMC / Shakhov / rescale -> Step 5 sums -> Step 2 free flight of the
 //      next interval, new key and histogram;
 //   2. reservoir injection at inflow faces (count, scan, write);
 //   3. exclusive scan of the histogram -> cell offsets of the new state;
 //   4. bookkeeping (particle count, Delta t of the next step, step index);
 //   5. scatter of source indices into the new cell order (the histogram is
-//      the cursor and ends at zero, ready for the next step).
+//      the cursor and ends at zero, ready for the next step), and in
+//      reproducible runs the source order inside each cell.
 // The sequence is captured once per buffer parity as a CUDA graph and
 // replayed by sp_step().
 #include <algorithm>
@@ -22,11 +23,6 @@
 
 #include "../../include/sp.h"
 #include "sp_internal.h"
-
-namespace sp {
-// Sort each cell's perm segment ascending (sp_noalloc.cu).
-void launch_order_cells(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s);
-}  // namespace sp
 
 using namespace sp;
 
@@ -463,7 +459,6 @@ StepArgs make_step_args(sp_ctx* c, int par) {
   a.cap = c->cap;
   a.big_cap = kHugeCell;
   a.cap_small = c->sched_cap;
-  a.stable = c->stable;
   a.surf = c->n_surf_tot > 0 ? c->surf : nullptr;
   a.one = c->n_inst == 1 ? 1 : 0;
   a.P0 = c->hP[0];
@@ -577,6 +572,14 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
                        c->surf_time, c->cyc, c->stream); ++n;
   rec(3);
   launch_scatter(c->key, c->start, c->count, c->perm, c->Mtot, c->cap, c->stream); ++n;
+  if (c->stable) {  // small and large cells side by side
+    cudaEventRecord(c->fork3_ev, c->stream);
+    cudaStreamWaitEvent(c->side2, c->fork3_ev, 0);
+    launch_order_large(c->start, c->NC, c->perm, c->side2); ++n;
+    cudaEventRecord(c->join2_ev, c->side2);
+    launch_order_small(c->start, c->NC, c->perm, c->stream); ++n;
+    cudaStreamWaitEvent(c->stream, c->join2_ev, 0);
+  }
   rec(4);
   return n;
 }
@@ -726,7 +729,7 @@ sp_status host_starts(sp_ctx* c, int inst, std::vector<uint32_t>& st) {
 }
 
 // perm over an instance's range, each cell's entries in ascending order
-// (the stable order the collision kernel restores).
+// (the order of reproducible runs).
 sp_status host_perm_sorted(sp_ctx* c, const std::vector<uint32_t>& st, std::vector<uint32_t>& pm) {
   const int64_t s0 = st[0], n = (int64_t)st.back() - s0;
   pm.resize(std::max<int64_t>(n, 1));
@@ -1051,6 +1054,12 @@ sp_status sp_set_reproducible(sp_ctx* c, int on) {
   if ((on != 0) != (c->stable != 0)) {
     c->stable = on != 0;
     destroy_graphs(c);
+    // the current state was left in scatter order: the next step and the
+    // moments expect the source order
+    if (c->stable && c->uploaded && !c->dirty) {
+      launch_order_cells(c->start, c->NC, c->perm, c->stream);
+      CK(cudaGetLastError());
+    }
   }
   return SP_OK;
 }
@@ -1170,7 +1179,6 @@ sp_status sp_moments(sp_ctx* c, int inst, int kind, double* out, int n_fields) {
       direct = (double*)pa.devicePointer;
     cudaGetLastError();  // (a pointer unknown to CUDA leaves an error to clear)
     if (direct) {
-      if (c->stable) launch_order_cells(c->start, c->NC, c->perm, c->stream);
       StepArgs a = make_step_args(c, c->cur);
       c->K->moments(a, P.cell_off, P.cell_off + nc, direct, c->stream);
       CK(cudaStreamSynchronize(c->stream));
@@ -1185,10 +1193,8 @@ sp_status sp_moments(sp_ctx* c, int inst, int kind, double* out, int n_fields) {
       c->mom_cells = nc;
     }
     double* d = c->mom;
-    // reproducible runs: each cell summed in source order (the scatter's
-    // order inside a cell is arbitrary; the collision step restores the
-    // same order, so this changes no later result)
-    if (c->stable) launch_order_cells(c->start, c->NC, c->perm, c->stream);
+    // (reproducible runs: every step leaves the cells in source order, so
+    // each cell is summed in that order)
     StepArgs a = make_step_args(c, c->cur);
     c->K->moments(a, P.cell_off, P.cell_off + nc, d, c->stream);
     CK(cudaMemcpyAsync(out, d, 8 * nf * nc, cudaMemcpyDeviceToHost, c->stream));

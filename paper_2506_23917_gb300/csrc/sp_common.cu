@@ -82,10 +82,13 @@ __global__ void k_scan_down(const uint32_t* in, uint32_t* out, int64_t n, const 
 }
 
 // perm[start[key] + rank] = source index.  The histogram itself is the
-// cursor: warp-aggregated atomic decrements hand out each cell's positions
-// from its end, and leave the histogram at zero for the next step's counts.
-// The order inside a cell is arbitrary here and restored to source order by
-// the collision kernel when the run is reproducible.
+// cursor: warp-aggregated atomic decrements leave it at zero for the next
+// step's counts, and count down to a cell's end, so that positions are handed
+// out from its beginning (start[key + 1] - the count before the decrement):
+// blocks run in about ascending order, and a cell fed by few of them often
+// arrives in source order.
+// The order inside a cell is arbitrary here; reproducible runs restore the
+// source order afterwards (k_order).
 constexpr int kScatterPer = 4;  // elements per thread, strided by the block size
 __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,
                           const uint32_t* Mtot, int64_t cap) {
@@ -104,17 +107,17 @@ __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* 
 #pragma unroll
   for (int j = 0; j < kScatterPer; ++j) {
     peers[j] = __match_any_sync(0xFFFFFFFFu, k[j]);
-    sk[j] = k[j] != kSentinel ? __ldg(&start[k[j]]) : 0u;
+    sk[j] = k[j] != kSentinel ? __ldg(&start[k[j] + 1]) : 0u;  // the cell's end
     base[j] = 0;
     if (k[j] != kSentinel && lane == __ffs(peers[j]) - 1)
-      base[j] = atomicSub(&count[k[j]], (uint32_t)__popc(peers[j])) - (uint32_t)__popc(peers[j]);
+      base[j] = atomicSub(&count[k[j]], (uint32_t)__popc(peers[j]));
   }
 #pragma unroll
   for (int j = 0; j < kScatterPer; ++j) {
     const uint32_t b = __shfl_sync(0xFFFFFFFFu, base[j], __ffs(peers[j]) - 1);
     if (k[j] != kSentinel) {
       const uint32_t rank = __popc(peers[j] & ((1u << lane) - 1u));
-      perm[sk[j] + b + rank] = (uint32_t)(i0 + (int64_t)j * blockDim.x);
+      perm[sk[j] - b + rank] = (uint32_t)(i0 + (int64_t)j * blockDim.x);
     }
   }
 }

@@ -678,12 +678,6 @@ __device__ __forceinline__ int64_t mesh_locate(const InstParams& P, const T* mfa
 // ---------------------------------------------------------------------------
 // Warp-cooperative pieces of the per-cell step.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int next_pow2(int n) {
-  int p = 1;
-  while (p < n) p <<= 1;
-  return p;
-}
-
 // Warp-aggregated histogram increment (key == kSentinel is skipped).
 __device__ __forceinline__ void warp_count(uint32_t key, uint32_t* count) {
   const unsigned peers = __match_any_sync(kFull, key);
@@ -1392,7 +1386,7 @@ __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, 
 
 // ---------------------------------------------------------------------------
 // One batch of G consecutive cells [k0, k0+G) whose particles fit the warp's
-// staging area: gather in stable order -> Step 3 moments -> Step 4 split,
+// staging area: gather through perm -> Step 3 moments -> Step 4 split,
 // DSMC, Shakhov, rescale -> Step 5 sums -> Step 2 free flight, new key and
 // histogram.  Particle work is spread over the lanes across the whole
 // batch; per-cell FP64 arithmetic runs lane-per-cell (lane i <-> cell i).
@@ -1431,7 +1425,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   __syncwarp();
   // the lanes' parts of the per-cell sums (split cells: FP32 state only)
   const auto lp = lane_parts<kSplitOf<T, DIM>>(ct, G, own, offi, Ni);
-  // ---- 1. source indices, cell of each slot, stable order within cells
+  // ---- 1. source indices (in source order within each cell when the run is
+  // reproducible: k_order) and cell of each slot
   // (the index copies run while the cell of each slot is written)
 #pragma unroll 4
   for (int s = lane; s < M; s += 32) cp_async<4>(&sidx[s], &a.perm[p0 + s]);
@@ -1447,62 +1442,6 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   }
   cp_async_wait_all();
   __syncwarp();
-  // cells whose source indices arrived out of order (the scatter's atomics
-  // keep only each scattering warp's run ascending); skipped when the run
-  // does not ask for the reproducible (source) order
-  unsigned mine_uns = 0;
-  if (a.stable)
-    for (int t = lane; t < M; t += 32) {
-      const int c = sseg[t];
-      if (t + 1 < ct->off[c + 1] && sidx[t] > sidx[t + 1]) mine_uns |= 1u << c;
-    }
-  const unsigned uns = __reduce_or_sync(kFull, mine_uns);
-  // small cells: each slot's rank among its cell's (distinct) source
-  // indices, written through the (not yet gathered) y-velocity array as
-  // scratch; big cells: a sorting network
-  const unsigned uns_big = __ballot_sync(kFull, ((uns >> lane) & 1u) && Ni > 64);
-  const unsigned uns_small = uns & ~uns_big;
-  if (uns_small) {
-    for (int s = lane; s < M; s += 32) {
-      const int c = sseg[s];
-      if (!((uns_small >> c) & 1u)) continue;
-      const int lo = ct->off[c], hi = ct->off[c + 1];
-      const uint32_t v = sidx[s];
-      int r = 0;
-      for (int j = lo; j < hi; ++j) r += sidx[j] < v;
-      ((uint32_t*)svy)[lo + r] = v;
-    }
-    __syncwarp();
-    for (int s = lane; s < M; s += 32)
-      if ((uns_small >> sseg[s]) & 1u) sidx[s] = ((const uint32_t*)svy)[s];
-    __syncwarp();
-  }
-  if (uns_big) {
-    const int nmax = __reduce_max_sync(kFull, ((uns_big >> lane) & 1u) ? (unsigned)Ni : 0u);
-    const int n2 = next_pow2(nmax);
-    // sorting network with all comparators pointing up: sorts a segment of
-    // any length in place (slots past its end act as +infinity)
-    for (int k = 2; k <= n2; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (unsigned rem = uns_big; rem; rem &= rem - 1) {
-          const int c = __ffs(rem) - 1;
-          const int lo = ct->off[c], n = ct->off[c + 1] - lo;
-          if (k > 2 * n) continue;  // every comparator of this stage is out of range
-          for (int li = lane; li < n; li += 32) {
-            const int q = (j == (k >> 1)) ? (li ^ (k - 1)) : (li ^ j);
-            if (q > li && q < n) {
-              const uint32_t x = sidx[lo + li], y = sidx[lo + q];
-              if (x > y) {
-                sidx[lo + li] = y;
-                sidx[lo + q] = x;
-              }
-            }
-          }
-        }
-        __syncwarp();
-      }
-    }
-  }
   // ---- 1b. Bird's sub-cells (option): each cell's slots in a stable order
   // by sub-cell (the sub-cell of a slot from its particle's position), so
   // that every sub-cell is a run of slots; offsets in ct->soff
@@ -1537,10 +1476,10 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     __syncwarp();
   }
   // the free flight re-reads the source indices from perm when they share
-  // the x-velocity array: store the restored (and sub-cell) order there
-  if (idx_in_velocity<T>() && (uns | subs)) {
+  // the x-velocity array: store the sub-cell order there
+  if (idx_in_velocity<T>() && subs) {
     for (int s = lane; s < M; s += 32)
-      if (((uns | subs) >> sseg[s]) & 1u) a.perm[p0 + s] = sidx[s];
+      if ((subs >> sseg[s]) & 1u) a.perm[p0 + s] = sidx[s];
   }
   // ---- 2. gather velocities (with the indices in the x-velocity array,
   // each lane reads slot s's index before it writes slot s's velocity)
@@ -2522,7 +2461,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, 1) k_collide(StepArgs 
 // the B velocity arrays, source indices in the key array, clash tags in the
 // first B position array; the free flight overwrites all three last), so
 // no cell size is refused.  The steps are those of process_batch for one
-// cell: stable order, gather, two-pass moments, cell_math, the NTC loop
+// cell: gather, two-pass moments, cell_math, the NTC loop
 // with exactly the one-by-one outcome (candidates of a round evaluated as
 // soon as their pair is final, decided against the prefix maximum of
 // sigma c), Shakhov resampling, the conservation rescale, Step 5 sums and
@@ -2604,28 +2543,6 @@ __device__ __forceinline__ void block_sums(TabT* tb, int n, typename Acc::result
   __syncthreads();
 }
 
-// In-place sorting network whose comparators all point one way, over n
-// slots by the whole block (slots past n act as +infinity).
-__device__ __forceinline__ void block_sort_u32(uint32_t* p, int n) {
-  int n2 = 1;
-  while (n2 < n) n2 <<= 1;
-  for (int k = 2; k <= n2; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < n; t += kHugeThreads) {
-        const int q = (j == (k >> 1)) ? (t ^ (k - 1)) : (t ^ j);
-        if (q > t && q < n) {
-          const uint32_t x = p[t], y = p[q];
-          if (x > y) {
-            p[t] = y;
-            p[q] = x;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-}
-
 template <class T, class A, int DIM, bool ONE, bool MESH = false>
 __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
   using Acc = CellAcc<T, A>;
@@ -2662,14 +2579,9 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
       sidx = a.key + p0;
       stag = (int*)((T*)a.Bpos[0] + p0);
     }
-    // ---- 1. source indices in stable (source) order
+    // ---- 1. source indices (in source order when the run is reproducible)
     for (int s = tid; s < N; s += kHugeThreads) sidx[s] = a.perm[p0 + s];
     __syncthreads();
-    if (a.stable) {
-      int uns = 0;
-      for (int s = tid; s + 1 < N; s += kHugeThreads) uns |= sidx[s] > sidx[s + 1];
-      if (__syncthreads_or(uns)) block_sort_u32(sidx, N);
-    }
     // Bird's sub-cells (option): the slots in a stable order by sub-cell
     const int nsub = Pi.nsub;
     if (nsub > 1) {

@@ -120,7 +120,7 @@ struct StepArgs {
   void* Bpos[3];
   void* Bvel[3];
   uint32_t* key;        // [cap]   key of each B slot
-  uint32_t* perm;       // [cap]   slot -> source index in A (FP32: sorted in place per cell)
+  uint32_t* perm;       // [cap]   slot -> source index in A (sub-cells, FP32: re-ordered in place)
   const uint32_t* start;// [NC+1]  cell offsets of the current state
   uint32_t* count;      // [NC]    next-state histogram (atomics)
   const uint32_t* cell_inst;  // [NC]
@@ -149,7 +149,6 @@ struct StepArgs {
   int64_t cap;
   int big_cap;          // staging capacity of the big-cell launch
   int cap_small;        // staging capacity per warp of the main launch
-  int stable;           // restore source order within cells (reproducible runs)
   double* surf;         // [elements][kSurfFields] wall tallies
   int one;              // a single instance: P0 is its parameter set
   // body-fitted O-grid instances (mesh = 1; all instances of a context
@@ -226,5 +225,11 @@ void launch_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
                           uint32_t* big_count, uint32_t* ticket, uint32_t* nbatch,
                           double* surf_time, unsigned long long* cyc, cudaStream_t s);
 int64_t scan_partial_size(int64_t n);
+
+// Each cell's perm segment in ascending (source) order (sp_noalloc.cu); the
+// small (up to 128 entries) and large cells separately, or both.
+void launch_order_small(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s);
+void launch_order_large(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s);
+void launch_order_cells(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s);
 
 }  // namespace sp

@@ -21,8 +21,8 @@ constexpr int64_t kStaticMaxKeys = int64_t(1) << 30;   // keys per call
 constexpr int64_t kStaticPartial = (kStaticMaxCells + 2047) / 2048 + 1;
 constexpr int kMaxDevices = 64;
 
-// [0, MAX): histogram, [MAX, 2 MAX): scatter cursors, then scan partials.
-static __device__ __align__(256) uint32_t g_sort_scratch[2 * kStaticMaxCells + kStaticPartial];
+// [0, MAX): histogram (also the scatter's cursors), then scan partials.
+static __device__ __align__(256) uint32_t g_sort_scratch[kStaticMaxCells + kStaticPartial];
 
 uint32_t* g_scratch_ptr[kMaxDevices] = {nullptr};
 
@@ -31,20 +31,55 @@ __global__ void k_static_zero(uint32_t* a, int64_t n) {
     a[i] = 0;
 }
 
-__global__ void k_static_hist(const uint32_t* key, int64_t n, int64_t ncells, uint32_t* count) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t k = key[i];
-  if (k < (uint64_t)ncells) atomicAdd(&count[k], 1u);
+// Keys come mostly in cell order (a moved state), so a warp's 32 keys hold a
+// few cells: one atomic per cell and warp, and kStaticPer keys per thread
+// whose load -> match -> atomic -> store chains overlap.
+constexpr int kStaticPer = 4;
+constexpr int kStaticThreads = 256;
+
+__global__ void __launch_bounds__(kStaticThreads) k_static_hist(const uint32_t* key, int64_t n, int64_t ncells,
+                                                                uint32_t* count) {
+  const int64_t i0 = (int64_t)blockIdx.x * kStaticThreads * kStaticPer + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  uint32_t k[kStaticPer];
+#pragma unroll
+  for (int j = 0; j < kStaticPer; ++j) {
+    const int64_t i = i0 + (int64_t)j * kStaticThreads;
+    k[j] = i < n ? key[i] : kSentinel;
+  }
+#pragma unroll
+  for (int j = 0; j < kStaticPer; ++j) {
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, k[j]);
+    if (k[j] < (uint64_t)ncells && lane == __ffs(peers) - 1) atomicAdd(&count[k[j]], (uint32_t)__popc(peers));
+  }
 }
 
-__global__ void k_static_scatter(const uint32_t* key, int64_t n, int64_t ncells, const uint32_t* start,
-                                 uint32_t* fill, uint32_t* perm) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t k = key[i];
-  if (k >= (uint64_t)ncells) return;
-  perm[start[k] + atomicAdd(&fill[k], 1u)] = (uint32_t)i;
+// The histogram is the cursor: it counts down to each cell's end.
+__global__ void __launch_bounds__(kStaticThreads) k_static_scatter(const uint32_t* key, int64_t n, int64_t ncells,
+                                                                   const uint32_t* start, uint32_t* count,
+                                                                   uint32_t* perm) {
+  const int64_t i0 = (int64_t)blockIdx.x * kStaticThreads * kStaticPer + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  uint32_t k[kStaticPer], at[kStaticPer];
+  unsigned peers[kStaticPer];
+#pragma unroll
+  for (int j = 0; j < kStaticPer; ++j) {
+    const int64_t i = i0 + (int64_t)j * kStaticThreads;
+    k[j] = i < n ? key[i] : kSentinel;
+  }
+#pragma unroll
+  for (int j = 0; j < kStaticPer; ++j) {
+    peers[j] = __match_any_sync(0xFFFFFFFFu, k[j]);
+    at[j] = 0;
+    if (k[j] < (uint64_t)ncells && lane == __ffs(peers[j]) - 1)
+      at[j] = start[(int64_t)k[j] + 1] - atomicSub(&count[k[j]], (uint32_t)__popc(peers[j]));
+  }
+#pragma unroll
+  for (int j = 0; j < kStaticPer; ++j) {
+    const uint32_t b = __shfl_sync(0xFFFFFFFFu, at[j], __ffs(peers[j]) - 1);
+    if (k[j] < (uint64_t)ncells)
+      perm[b + __popc(peers[j] & ((1u << lane) - 1u))] = (uint32_t)(i0 + (int64_t)j * kStaticThreads);
+  }
 }
 
 // In-place sorting network whose comparators all point the same way (each
@@ -75,43 +110,248 @@ __device__ __forceinline__ void sort_segment(uint32_t* p, int64_t n, int64_t tid
   }
 }
 
-// Segments of at most kWarpSeg entries: one warp each.
-constexpr int64_t kWarpSeg = 1024;
-// Larger segments: one block of kOrderThreads threads each, staged in shared
-// memory up to kSmemSeg entries, else sorted in place in global memory
-// (L2-resident for the segment sizes a cell reaches; a segment of 2^20
-// entries takes a few tenths of a second).
-constexpr int kOrderThreads = 512;
-constexpr int kSmemSeg = 8192;
+// Stable order of the cells' entries.  The scatter's atomics leave each
+// cell's source indices in arbitrary order; two kernels over disjoint cell
+// sizes put them in ascending order:
+//   k_order_small  up to kSmallSeg: one warp per cell, up to 4 entries per lane;
+//   k_order_large  to kWarpSeg: one warp per cell, 8 to 32 entries per lane;
+//                  above: one block per cell.
+// Bound by the issue of the shuffles and compares, about 3 warp-instructions
+// per entry, at full occupancy and without shared memory for small cells.
+// 600 x 300 cylinder (6.6 M entries, 40 per cell): 53 us; sphere, 30 M
+// entries, 1 M cells: 0.21 ms; jet, 4.5 M entries, most in cells of 500 to
+// 2000: 74 us.  Restoring the order inside the collision kernel instead (12
+// resident warps per SM, one shared-memory read per comparison) took 0.15,
+// 0.38 and 0.38 ms of those flows' steps.
+constexpr int kSmallSeg = 128;
+constexpr int kWarpSeg = 1024;
+constexpr int kSmemSeg = 8192;       // big cells up to this size are staged in shared memory
+constexpr int kOrderWarps = 8;
+constexpr int kOrderThreads = 32 * kOrderWarps;
+constexpr int kOrderSmem = kSmemSeg + kSmemSeg / 32;  // words: a pad word every 32
 
-__global__ void k_static_order(const uint32_t* start, int64_t ncells, uint32_t* perm) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < ncells; c += nw) {
-    const uint32_t s0 = start[c];
-    const int64_t n = (int64_t)start[c + 1] - (int64_t)s0;
-    if (n < 2 || n > kWarpSeg) continue;
-    sort_segment(perm + s0, n, lane, 32, [] { __syncwarp(); });
+__device__ __forceinline__ void lo_hi(uint32_t& a, uint32_t& b) {
+  const uint32_t x = a < b ? a : b, y = a < b ? b : a;
+  a = x;
+  b = y;
+}
+
+// Ascending sort of 32 R entries held by a warp, entry lane R + i in x[i]
+// (any assignment of the input to lanes will do): the network of
+// sort_segment, with the stages inside a lane on registers and the others
+// by shuffles.
+template <int R>
+__device__ __forceinline__ void warp_sort(uint32_t (&x)[R], int lane) {
+#pragma unroll
+  for (int k = 2; k <= R; k <<= 1) {
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+      if ((i ^ (k - 1)) > i) lo_hi(x[i], x[i ^ (k - 1)]);
+#pragma unroll
+    for (int j = k >> 2; j > 0; j >>= 1)
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (!(i & j)) lo_hi(x[i], x[i | j]);
+  }
+#pragma unroll 1
+  for (int kl = 2; kl <= 32; kl <<= 1) {
+    const bool lo = !(lane & (kl >> 1));
+    if constexpr (R == 1) {
+      const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[0], kl - 1);
+      x[0] = (x[0] < y) == lo ? x[0] : y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < R / 2; ++i) {
+        const uint32_t y0 = __shfl_xor_sync(0xFFFFFFFFu, x[R - 1 - i], kl - 1);
+        const uint32_t y1 = __shfl_xor_sync(0xFFFFFFFFu, x[i], kl - 1);
+        x[i] = (x[i] < y0) == lo ? x[i] : y0;
+        x[R - 1 - i] = (x[R - 1 - i] < y1) == lo ? x[R - 1 - i] : y1;
+      }
+    }
+#pragma unroll 1
+    for (int m = kl >> 2; m > 0; m >>= 1) {
+      const bool up = !(lane & m);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[i], m);
+        x[i] = (x[i] < y) == up ? x[i] : y;
+      }
+    }
+#pragma unroll
+    for (int j = R / 2; j > 0; j >>= 1)
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (!(i & j)) lo_hi(x[i], x[i | j]);
   }
 }
 
-__global__ void __launch_bounds__(kOrderThreads) k_static_order_big(const uint32_t* start, int64_t ncells,
-                                                                     uint32_t* perm) {
-  __shared__ uint32_t sh[kSmemSeg];
-  for (int64_t c = blockIdx.x; c < ncells; c += gridDim.x) {
-    const uint32_t s0 = start[c];
-    const int64_t n = (int64_t)start[c + 1] - (int64_t)s0;
-    if (n <= kWarpSeg) continue;
-    uint32_t* g = perm + s0;
-    if (n <= kSmemSeg) {
-      for (int64_t t = threadIdx.x; t < n; t += blockDim.x) sh[t] = g[t];
-      __syncthreads();
-      sort_segment(sh, n, threadIdx.x, blockDim.x, [] { __syncthreads(); });
-      for (int64_t t = threadIdx.x; t < n; t += blockDim.x) g[t] = sh[t];
-    } else {
-      sort_segment(g, n, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+// The entries x (entry 32 i + lane in x[i], 0xFFFFFFFF past the end) of one
+// cell p[0..n), n <= 32 R, put in order and stored, unless they are in order
+// already.  A lane's sorted entries are consecutive, so above R = 4 the
+// stores go through the warp's shared memory.
+template <int R>
+__device__ __forceinline__ void order_entries(uint32_t (&x)[R], uint32_t* p, int n, int lane, uint32_t* sh) {
+  bool asc = true;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {  // against the next entry (lane 31: the next row's first)
+    uint32_t nx = __shfl_sync(0xFFFFFFFFu, x[i], (lane + 1) & 31);
+    if (i + 1 < R) {
+      const uint32_t f = __shfl_sync(0xFFFFFFFFu, x[i + 1 < R ? i + 1 : i], 0);
+      if (lane == 31) nx = f;
+    } else if (lane == 31) {
+      nx = 0xFFFFFFFFu;
     }
-    __syncthreads();
+    asc = asc && x[i] <= nx;
+  }
+  if (__all_sync(0xFFFFFFFFu, asc)) return;
+  warp_sort<R>(x, lane);
+  if constexpr (R <= 4) {
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+      if (lane * R + i < n) p[lane * R + i] = x[i];
+  } else {
+    constexpr int S = 32 + 32 / R;  // row length: no bank conflicts either way
+#pragma unroll
+    for (int i = 0; i < R; ++i) sh[i * S + lane] = x[i];
+    __syncwarp();
+    for (int t = lane; t < n; t += 32) p[t] = sh[(t % R) * S + t / R];
+    __syncwarp();
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void order_cell(uint32_t* p, int n, int lane, uint32_t* sh) {
+  uint32_t x[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) x[i] = 32 * i + lane < n ? p[32 * i + lane] : 0xFFFFFFFFu;
+  order_entries<R>(x, p, n, lane, sh);
+}
+
+// A cell of n <= 8 * 32 R entries by the whole block: warp w sorts entries
+// [32 R w, 32 R (w + 1)) in its registers, then every entry finds its place
+// by binary searches in the other runs (the entries are distinct).
+template <int R>
+__device__ __forceinline__ void order_block(uint32_t* g, int n, uint32_t* seg) {
+  constexpr int L = 32 * R;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const auto pad = [](int e) { return e + (e >> 5); };
+  if (L * w < n) {
+    uint32_t x[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int t = L * w + 32 * i + lane;
+      x[i] = t < n ? g[t] : 0xFFFFFFFFu;
+    }
+    warp_sort<R>(x, lane);
+#pragma unroll
+    for (int i = 0; i < R; ++i) seg[pad(L * w + R * lane + i)] = x[i];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < n; t += kOrderThreads) {
+    const uint32_t v = seg[pad(t)];
+    // the runs' counts of entries below v, searched side by side (its own
+    // run's is its place there; the last run is padded with the largest value)
+    int lo[kOrderWarps];
+#pragma unroll
+    for (int r = 0; r < kOrderWarps; ++r) lo[r] = 0;
+#pragma unroll
+    for (int h = L / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int r = 0; r < kOrderWarps; ++r)
+        if (L * r < n && seg[pad(L * r + lo[r] + h - 1)] < v) lo[r] += h;
+    int at = 0;
+#pragma unroll
+    for (int r = 0; r < kOrderWarps; ++r)
+      if (L * r < n) at += lo[r] + (seg[pad(L * r + lo[r])] < v ? 1 : 0);
+    g[at] = v;
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void order_big_cell(uint32_t* g, int64_t n, uint32_t* seg) {
+  static_assert(kSmemSeg == kOrderWarps * 1024 && kWarpSeg < kOrderWarps * 256, "runs of one warp each");
+  if (n <= kOrderWarps * 256) order_block<8>(g, (int)n, seg);
+  else if (n <= kOrderWarps * 512) order_block<16>(g, (int)n, seg);
+  else if (n <= kSmemSeg) order_block<32>(g, (int)n, seg);
+  else sort_segment(g, n, threadIdx.x, kOrderThreads, [] { __syncthreads(); });
+}
+
+// Cells up to kSmallSeg entries: a warp takes kOrderCells consecutive cells
+// and requests the entries of all of them (up to 64 each) before it sorts the
+// first, so that one round trip to memory serves them together.
+constexpr int kOrderCells = 4;
+__global__ void __launch_bounds__(kOrderThreads, 6) k_order_small(const uint32_t* start, int64_t ncells,
+                                                                  uint32_t* perm) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = (int64_t)gridDim.x * kOrderWarps;
+  for (int64_t c0 = ((int64_t)blockIdx.x * kOrderWarps + (threadIdx.x >> 5)) * kOrderCells; c0 < ncells;
+       c0 += nw * kOrderCells) {
+    const int64_t at = c0 + (lane <= kOrderCells ? lane : kOrderCells);
+    const uint32_t sl = start[at < ncells ? at : ncells];
+    uint32_t x[kOrderCells][2];
+#pragma unroll
+    for (int j = 0; j < kOrderCells; ++j) {
+      const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, sl, j), n = __shfl_sync(0xFFFFFFFFu, sl, j + 1) - s0;
+      const uint32_t m = n <= 64 ? n : 0;
+      x[j][0] = (uint32_t)lane < m ? perm[s0 + lane] : 0xFFFFFFFFu;
+      x[j][1] = (uint32_t)lane + 32 < m ? perm[s0 + lane + 32] : 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int j = 0; j < kOrderCells; ++j) {
+      const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, sl, j), n = __shfl_sync(0xFFFFFFFFu, sl, j + 1) - s0;
+      if (n < 2 || n > (uint32_t)kSmallSeg) continue;
+      if (n <= 32) {
+        uint32_t y[1] = {x[j][0]};
+        order_entries<1>(y, perm + s0, (int)n, lane, nullptr);
+      } else if (n <= 64) {
+        order_entries<2>(x[j], perm + s0, (int)n, lane, nullptr);
+      } else {
+        order_cell<4>(perm + s0, (int)n, lane, nullptr);
+      }
+    }
+  }
+}
+
+// Larger cells.  Blocks [0, gb) take those above kWarpSeg, the others the
+// rest.  The cells are dealt out with the stride of all takers (thread or
+// lane t of taker b looks at cell b + t stride), so that a region of dense
+// cells is spread over many of them.
+__global__ void __launch_bounds__(kOrderThreads, 4) k_order_large(const uint32_t* start, int64_t ncells,
+                                                                  uint32_t* perm, unsigned gb) {
+  __shared__ uint32_t sh[kOrderSmem];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (blockIdx.x >= gb) {
+    uint32_t* ws = sh + w * (kOrderSmem / kOrderWarps);
+    const int64_t nw = (int64_t)(gridDim.x - gb) * kOrderWarps;
+    for (int64_t cb = (int64_t)(blockIdx.x - gb) * kOrderWarps + w; cb < ncells; cb += 32 * nw) {
+      const int64_t c = cb + (int64_t)lane * nw;
+      const uint32_t s0 = c < ncells ? start[c] : 0u, n = c < ncells ? start[c + 1] - s0 : 0u;
+      for (unsigned todo = __ballot_sync(0xFFFFFFFFu, n > (uint32_t)kSmallSeg && n <= (uint32_t)kWarpSeg); todo;
+           todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        uint32_t* p = perm + __shfl_sync(0xFFFFFFFFu, s0, src);
+        const int m = (int)__shfl_sync(0xFFFFFFFFu, n, src);
+        if (m <= 256) order_cell<8>(p, m, lane, ws);
+        else if (m <= 512) order_cell<16>(p, m, lane, ws);
+        else order_cell<32>(p, m, lane, ws);
+      }
+    }
+  } else {
+    __shared__ uint32_t list[kOrderThreads];
+    __shared__ int nlist;
+    for (int64_t cb = blockIdx.x; cb < ncells; cb += (int64_t)kOrderThreads * gb) {
+      if (threadIdx.x == 0) nlist = 0;
+      __syncthreads();
+      const int64_t c = cb + (int64_t)threadIdx.x * gb;
+      if (c < ncells && start[c + 1] - start[c] > (uint32_t)kWarpSeg) list[atomicAdd(&nlist, 1)] = (uint32_t)c;
+      __syncthreads();
+      const int nl = nlist;
+      for (int q = 0; q < nl; ++q) {
+        const int64_t k = (int64_t)list[q];
+        order_big_cell(perm + start[k], (int64_t)(start[k + 1] - start[k]), sh);
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -134,15 +374,26 @@ cudaError_t static_scratch(uint32_t** out) {
 
 }  // namespace
 
-// Each cell's permutation entries put in ascending (source) order: a warp
-// per cell up to kWarpSeg entries, a block per larger cell.
-void launch_order_cells(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s) {
+// Each cell's permutation entries put in ascending (source) order: the two
+// launches touch disjoint cells and may run side by side.
+void launch_order_small(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s) {
   if (ncells <= 0) return;
-  int64_t ob = (ncells + 7) / 8;
-  if (ob > 8192) ob = 8192;
-  k_static_order<<<(unsigned)ob, 256, 0, s>>>(start, ncells, perm);
-  const int64_t bb = ncells < 1024 ? ncells : 1024;
-  k_static_order_big<<<(unsigned)bb, kOrderThreads, 0, s>>>(start, ncells, perm);
+  int64_t g = (ncells + kOrderWarps * kOrderCells - 1) / (kOrderWarps * kOrderCells);
+  if (g > (int64_t(1) << 20)) g = int64_t(1) << 20;
+  k_order_small<<<(unsigned)g, kOrderThreads, 0, s>>>(start, ncells, perm);
+}
+
+void launch_order_large(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s) {
+  if (ncells <= 0) return;
+  const int64_t gb = ncells < 608 ? ncells : 608;
+  int64_t gm = (ncells + 8 * kOrderWarps - 1) / (8 * kOrderWarps);  // (about 8 cells to look at per warp)
+  if (gm > 4096) gm = 4096;
+  k_order_large<<<(unsigned)(gb + gm), kOrderThreads, 0, s>>>(start, ncells, perm, (unsigned)gb);
+}
+
+void launch_order_cells(const uint32_t* start, int64_t ncells, uint32_t* perm, cudaStream_t s) {
+  launch_order_large(start, ncells, perm, s);
+  launch_order_small(start, ncells, perm, s);
 }
 
 }  // namespace sp
@@ -169,17 +420,15 @@ extern "C" sp_status sp_sort_cells_static(const uint32_t* d_keys, int64_t n, int
   }
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t* count = scratch;
-  uint32_t* fill = scratch + kStaticMaxCells;
-  uint32_t* partial = scratch + 2 * kStaticMaxCells;
-  // the array keeps the previous call's contents: both counters restart at 0
+  uint32_t* partial = scratch + kStaticMaxCells;
+  // the array keeps the previous call's contents: the counters restart at 0
   int64_t zb = (ncells + 255) / 256;
   if (zb > 4096) zb = 4096;
   k_static_zero<<<(unsigned)zb, 256, 0, s>>>(count, ncells);
-  k_static_zero<<<(unsigned)zb, 256, 0, s>>>(fill, ncells);
-  const unsigned nb = (unsigned)((n + 255) / 256);
-  if (n > 0) k_static_hist<<<nb, 256, 0, s>>>(d_keys, n, ncells, count);
+  const unsigned nb = (unsigned)((n + kStaticThreads * kStaticPer - 1) / (kStaticThreads * kStaticPer));
+  if (n > 0) k_static_hist<<<nb, kStaticThreads, 0, s>>>(d_keys, n, ncells, count);
   launch_scan(count, d_start, ncells, partial, s);
-  if (n > 0) k_static_scatter<<<nb, 256, 0, s>>>(d_keys, n, ncells, d_start, fill, d_perm);
+  if (n > 0) k_static_scatter<<<nb, kStaticThreads, 0, s>>>(d_keys, n, ncells, d_start, count, d_perm);
   launch_order_cells(d_start, ncells, d_perm, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
