@@ -44,7 +44,8 @@ struct sp_ctx {
   // device buffers
   void* pos[2][3] = {{nullptr}};
   void* vel[2][3] = {{nullptr}};
-  uint32_t *key = nullptr, *perm = nullptr, *count = nullptr, *start = nullptr;
+  uint32_t* key[2] = {nullptr, nullptr};  // cell of each slot of the particle buffers
+  uint32_t *perm = nullptr, *count = nullptr, *start = nullptr;
   uint32_t *cell_inst = nullptr, *scan_part = nullptr, *big_list = nullptr, *big_count = nullptr;
   uint32_t* ticket = nullptr;
   uint2* batches = nullptr;
@@ -422,7 +423,8 @@ StepArgs make_step_args(sp_ctx* c, int par) {
     a.Avel[d] = c->vel[par][d];
     a.Bvel[d] = c->vel[1 - par][d];
   }
-  a.key = c->key;
+  a.key_in = c->key[par];
+  a.key = c->key[1 - par];
   a.perm = c->perm;
   a.start = c->start;
   a.count = c->count;
@@ -476,7 +478,7 @@ InjectArgs make_inject_args(sp_ctx* c, int par) {
     a.Bpos[d] = c->pos[1 - par][d];
     a.Bvel[d] = c->vel[1 - par][d];
   }
-  a.key = c->key;
+  a.key = c->key[1 - par];
   a.count = c->count;
   a.P = c->dP;
   a.dt_cur = c->dt_cur;
@@ -511,7 +513,7 @@ bool apply_schedule(sp_ctx* c, int cap, int warps) {
   const size_t smem = c->K->collide_smem(warps, cap);
   if (smem > (size_t)kMaxDynSmem) return false;
   const bool one = c->n_inst == 1;
-  const int per_sm = c->K->collide_blocks_per_sm(c->dim, warps, cap, one, c->mesh != 0);
+  const int per_sm = c->K->collide_blocks_per_sm(c->dim, warps, cap, one);
   if (per_sm < 1) return false;
   c->sched_cap = cap;
   c->sched_warps = warps;
@@ -563,6 +565,7 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   launch_collide_p(c, a, false, small_grid(c), c->stream); ++n;
   cudaStreamWaitEvent(c->stream, c->join2_ev, 0);
   cudaStreamWaitEvent(c->stream, c->join3_ev, 0);
+  c->K->flight(c->dim, a, c->nsm, c->stream); ++n;
   rec(1);
   if (fork) cudaStreamWaitEvent(c->stream, c->join_ev, 0);
   rec(2);
@@ -571,7 +574,7 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
                        c->NC, c->goff, c->gcount, c->n_ghost, c->big_count, c->ticket, c->nbatch,
                        c->surf_time, c->cyc, c->stream); ++n;
   rec(3);
-  launch_scatter(c->key, c->start, c->count, c->perm, c->Mtot, c->cap, c->stream); ++n;
+  launch_scatter(c->key[1 - par], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream); ++n;
   if (c->stable) {  // small and large cells side by side
     cudaEventRecord(c->fork3_ev, c->stream);
     cudaStreamWaitEvent(c->side2, c->fork3_ev, 0);
@@ -671,16 +674,16 @@ sp_status upload(sp_ctx* c) {
   CK(cudaMemsetAsync(c->count, 0, sizeof(uint32_t) * c->NC, c->stream));
   const void* P3[3] = {c->pos[c->cur][0], c->pos[c->cur][1], c->pos[c->cur][2]};
   if (c->mesh)
-    c->K->keys_mesh(P3, M, c->part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key, c->count, c->stream);
+    c->K->keys_mesh(P3, M, c->part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key[c->cur], c->count, c->stream);
   else
-    c->K->keys(dim, P3, M, c->part_inst, c->dP, c->key, c->count, c->stream);
+    c->K->keys(dim, P3, M, c->part_inst, c->dP, c->key[c->cur], c->count, c->stream);
   launch_scan(c->count, c->start, c->NC, c->scan_part, c->stream);
   c->hM = (uint32_t)M;
   CK(cudaMemcpyAsync(c->Mtot, &c->hM, 4, cudaMemcpyHostToDevice, c->stream));
   // the state holds the located particles only: an O-grid drops those
   // outside the mesh (sentinel keys), so its size is start[NC], not M
   CK(cudaMemcpyAsync(c->Mcur, c->start + c->NC, 4, cudaMemcpyDeviceToDevice, c->stream));
-  launch_scatter(c->key, c->start, c->count, c->perm, c->Mtot, c->cap, c->stream);
+  launch_scatter(c->key[c->cur], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream);
   // the scatter's atomics leave each cell's order arbitrary: reproducible
   // runs restore the source order, so that the moments below (and the first
   // step's Delta t) sum each cell in the same order on every run
@@ -824,7 +827,7 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
         if (d < dim) CK(dalloc(&c->pos[b][d], cap * c->tsize));
         CK(dalloc(&c->vel[b][d], cap * c->tsize));
       }
-    CK(dalloc(&c->key, 4 * cap));
+    for (int b = 0; b < 2; ++b) CK(dalloc(&c->key[b], 4 * cap));
     CK(dalloc(&c->part_inst, 4 * cap));
     CK(dalloc(&c->perm, 4 * cap));
     CK(dalloc(&c->count, 4 * NC));
@@ -1107,7 +1110,7 @@ sp_status sp_autotune(sp_ctx* c, int steps_per_trial, int* cap_out, int* warps_o
     for (int ci : caps) sched.push_back({ci, wi});
     int last = -1;
     for (int ci = kHugeCell; ci >= 128; ci -= 32) {
-      const int per = c->K->collide_blocks_per_sm(c->dim, wi, ci, c->n_inst == 1, c->mesh != 0);
+      const int per = c->K->collide_blocks_per_sm(c->dim, wi, ci, c->n_inst == 1);
       if (per != last && per > 0 &&
           std::find(sched.begin(), sched.end(), std::make_pair(ci, wi)) == sched.end())
         sched.push_back({ci, wi});
@@ -1456,7 +1459,7 @@ sp_status sp_free(sp_ctx* c) {
       cudaFree(c->vel[b][d]);
     }
   for (double* p : c->dstage) cudaFree(p);
-  void* ptrs[] = {c->Lc, c->iLc, c->mrad, c->mface, c->mnode, c->ivol, c->rcp, c->cons, c->mom, c->msum, c->cost, c->cyc, c->surf, c->surf_time, c->batches, c->nbatch, c->ticket, c->part_inst, c->key, c->perm, c->count, c->start, c->cell_inst, c->scan_part, c->big_list,
+  void* ptrs[] = {c->Lc, c->iLc, c->mrad, c->mface, c->mnode, c->ivol, c->rcp, c->cons, c->mom, c->msum, c->cost, c->cyc, c->surf, c->surf_time, c->batches, c->nbatch, c->ticket, c->part_inst, c->key[0], c->key[1], c->perm, c->count, c->start, c->cell_inst, c->scan_part, c->big_list,
                   c->big_count, c->vol, c->smax, c->rem, c->samp, c->rec, c->resamp, c->dP, c->dt_cur, c->dt_min,
                   c->step_d, c->Mcur, c->Mtot, c->err, c->ghosts, c->gcount, c->goff, c->gscan_part};
   for (void* p : ptrs) cudaFree(p);

@@ -321,12 +321,13 @@ __device__ __forceinline__ void diffuse_sample(T RTw, Uni<T>& r, T* cn, T* t1, T
   *t2 = s * sn * r4;
 }
 
-// FP32 free flight: whether the straight flight over trem stays inside the
-// box by the rounding margin and misses the body (the first test of
-// move_particle, without its square root and division: for a pair
-// approaching the body, t < trem <=> -b - trem a < sqrt(disc)); if so x is
-// moved to the end point.  Branch-free, so that two particles' tests
-// interleave.
+// Whether the straight flight over trem stays inside the box by the rounding
+// margin and misses the body (the first test of move_particle, without its
+// square root and division: for a particle approaching the body,
+// t < trem <=> -b - trem a < sqrt(disc)); if so x is moved to the end point.
+// In 2-D FP32 the comparison decides as it stands; elsewhere only a
+// particle that misses by a margin far above rounding is cleared, so that
+// move_particle's quotient decides every close case.
 template <class T, int DIM>
 __device__ __forceinline__ bool flight_fast(const InstParams& P, T* x, const T* v, T trem) {
   const Geo<T>& G = geo<T>(P);
@@ -349,8 +350,15 @@ __device__ __forceinline__ bool flight_fast(const InstParams& P, T* x, const T* 
     }
     cc -= G.body_r * G.body_r;
     const T disc = bb * bb - aa * cc;
-    const T q = -bb - trem * aa;
-    const bool hit = bb < (T)0 && aa > (T)0 && disc >= (T)0 && (q < (T)0 || q * q < disc);
+    T q = -bb - trem * aa;
+    bool hit;
+    if constexpr (sizeof(T) == 4 && DIM == 2) {
+      hit = bb < (T)0 && aa > (T)0 && disc >= (T)0 && (q < (T)0 || q * q < disc);
+    } else {
+      q += bb * (sizeof(T) == 4 ? (T)1e-5 : (T)1e-12);  // (b < 0: towards a hit)
+      hit = bb < (T)0 && aa > (T)0 && disc >= -(bb * bb) * (sizeof(T) == 4 ? (T)1e-5 : (T)1e-12) &&
+            (q < (T)0 || q * q < disc);
+    }
     ok = ok && !hit;
   }
   if (ok) {
@@ -850,16 +858,6 @@ __device__ __forceinline__ float2 acc_pair(const PlainSum<double>&) { return mak
 // the copy in the kernel's parameter space, so that the geometry and gas
 // constants reach the arithmetic as constant-bank operands rather than as
 // per-particle loads.
-// 32-slot rounds of the free flight whose positions are loaded together
-// (registers: rounds x DIM values of T)
-template <class T>
-constexpr int kFlightRounds = sizeof(T) == 4 ? 16 : 4;
-// FP32 rounds whose straight-flight tests are formed together: pairs in
-// 2-D (+10 % on the cylinder; groups of 4: +4 %, of 8: -9 %); 1-D and 3-D
-// keep one round at a time (pairs cost the 3-D sphere 10 %)
-template <int DIM>
-constexpr int kFlightGroup = DIM == 2 ? 2 : 1;
-
 template <bool ONE>
 __device__ __forceinline__ const InstParams& inst_params(const StepArgs& a, uint32_t i) {
   if constexpr (ONE) return a.P0;
@@ -1391,7 +1389,7 @@ __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, 
 // histogram.  Particle work is spread over the lanes across the whole
 // batch; per-cell FP64 arithmetic runs lane-per-cell (lane i <-> cell i).
 // ---------------------------------------------------------------------------
-template <class T, class A, int DIM, bool ONE, bool MESH = false>
+template <class T, class A, int DIM, bool ONE>
 __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A>* ct, uint32_t* sidx,
                               int* stag, uint8_t* sseg, T* svx, T* svy, T* svz) {
   using Acc = CellAcc<T, A>;
@@ -1475,29 +1473,25 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     }
     __syncwarp();
   }
-  // the free flight re-reads the source indices from perm when they share
-  // the x-velocity array: store the sub-cell order there
-  if (idx_in_velocity<T>() && subs) {
+  // the free flight reads the source indices from perm: store the sub-cell
+  // order there
+  if (subs) {
     for (int s = lane; s < M; s += 32)
       if ((subs >> sseg[s]) & 1u) a.perm[p0 + s] = sidx[s];
   }
   // ---- 2. gather velocities (with the indices in the x-velocity array,
-  // each lane reads slot s's index before it writes slot s's velocity)
+  // each lane reads slot s's index before it writes slot s's velocity);
+  // every lane issues all of its copies before waiting once
   {
     const T* Av0 = (const T*)a.Avel[0];
     const T* Av1 = (const T*)a.Avel[1];
     const T* Av2 = (const T*)a.Avel[2];
-    // every lane issues all of its copies before waiting once; the
-    // positions, read only by the free flight at the end of the batch, are
-    // requested into L2 now so that those reads do not wait on HBM
 #pragma unroll 4
     for (int s = lane; s < M; s += 32) {
       const uint32_t o = sidx[s];
       cp_async<sizeof(T)>(&svx[s], &Av0[o]);
       cp_async<sizeof(T)>(&svy[s], &Av1[o]);
       cp_async<sizeof(T)>(&svz[s], &Av2[o]);
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) prefetch_l2(&((const T*)a.Apos[d])[o]);
       stag[s] = 0x7FFFFFFF;
     }
     cp_async_wait_all();
@@ -1973,11 +1967,6 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     }
   }
   __syncwarp();
-  // FP32 staging: the free flight's source indices, copied from perm into
-  // the clash-tag array (free from here on) while the next phases run
-  if (idx_in_velocity<T>()) {
-    for (int s = lane; s < M; s += 32) cp_async<4>(&stag[s], &a.perm[p0 + s]);
-  }
   // ---- 7. conservation rescale c' = U + (c_p - U_p) sqrt(T/T_p) of every
   // particle of a cell with a resampled particle; U, T are the Step 3
   // moments (the targets), U_p, T_p those after the Shakhov sub-step.
@@ -2196,177 +2185,21 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       a.rec[3 * NC + kc] = ct->nar[lane];
     }
   }
-  // ---- 9. free flight of the next interval (Step 2), key and histogram;
-  // positions of kFlightRounds rounds are loaded before any is used, then the rounds
-  // run through one copy of the free-flight code (the loaded positions
-  // rotate through registers)
-  T* Bx[3] = {(T*)a.Bpos[0], (T*)a.Bpos[1], (T*)a.Bpos[2]};
-  T* Bv[3] = {(T*)a.Bvel[0], (T*)a.Bvel[1], (T*)a.Bvel[2]};
-  if (idx_in_velocity<T>()) cp_async_wait_all();
-  __syncwarp();
-  if constexpr (MESH) {
-    // body-fitted mesh: the walk from the particle's cell gives its next
-    // cell (point location by face crossing).  The face records of the
-    // batch's cells (12 values each) are staged in the table's per-cell
-    // arrays that are dead by now (U and q for cells 0-15, Up and Kl for
-    // 16-31), so that each particle's first walk step reads shared memory.
-    using CT = CellTab<T, A>;
-    static_assert(offsetof(CT, q) == offsetof(CT, U) + 96 * sizeof(T) &&
-                      offsetof(CT, Kl) == offsetof(CT, Up) + 96 * sizeof(T),
-                  "U, q and Up, Kl must each be 16 x 12 contiguous values");
-    T* fst0 = &ct->U[0][0];
-    T* fst1 = &ct->Up[0][0];
-    if (own) {
-      const T* src = (const T*)a.mface + 12 * kc;
-      T* dst = lane < 16 ? fst0 + 12 * lane : fst1 + 12 * (lane - 16);
-#pragma unroll
-      for (int e = 0; e < 12; ++e) dst[e] = src[e];
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int sb = 0; sb < M; sb += 32) {
-      const int s = sb + lane;
-      uint32_t key = kSentinel;
-      if (s < M) {
-        const int c = sseg[s];
-        const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-        const uint32_t o = idx_in_velocity<T>() ? (uint32_t)stag[s] : sidx[s];
-        T x[3] = {((const T*)a.Apos[0])[o], ((const T*)a.Apos[1])[o], (T)0};
-        T v[3] = {svx[s], svy[s], svz[s]};
-        int64_t kl = ct->kl[c];
-        const T* f0 = c < 16 ? fst0 + 12 * c : fst1 + 12 * (c - 16);
-        const bool gone = mesh_walk<T>(P, (const T*)a.mface, a.surf, kl, x, v, ct->dt[c], step, kPurpWall,
-                                       (uint32_t)ct->kl[c], (uint32_t)(s - ct->off[c]), 0u, a.err, false, f0);
-        if (!gone) key = (uint32_t)(P.cell_off + kl);
-        Bx[0][p0 + s] = x[0];
-        Bx[1][p0 + s] = x[1];
-        Bv[0][p0 + s] = v[0];
-        Bv[1][p0 + s] = v[1];
-        Bv[2][p0 + s] = v[2];
-        a.key[p0 + s] = key;
-      }
-      warp_count(key, a.count);
-    }
-    __syncwarp();
-    return;
-  }
-  constexpr int R = kFlightRounds<T>;
-  for (int sb0 = 0; sb0 < M; sb0 += 32 * R) {
-    T xr[R][DIM] = {};
-#pragma unroll
-    for (int u = 0; u < R; ++u) {
-      const int s = sb0 + 32 * u + lane;
-      if (s < M) {
-        const uint32_t o = idx_in_velocity<T>() ? (uint32_t)stag[s] : sidx[s];
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) xr[u][d] = ((const T*)a.Apos[d])[o];
-      }
-    }
-    if constexpr (sizeof(T) == 4 && kFlightGroup<DIM> > 1) {
-      // FP32: rounds in groups of W.  The straight-flight tests, end points
-      // and keys of the group are formed first, branch-free, so that their
-      // dependent chains interleave; then each round (the next rotated into
-      // the first registers: one copy of the code) stores its particles,
-      // running the full free flight for those the test did not clear.
-      constexpr int W = kFlightGroup<DIM>;
-#pragma unroll 1
-      for (int u = 0; u < R; u += W) {
-        const int sb = sb0 + 32 * u;
-        if (sb >= M) break;
-        int sg[W], cg[W];
-        bool okg[W], fg[W];
-        T xg[W][3], vg[W][3], dtg[W];
-        uint32_t kg[W];
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-          sg[j] = sb + 32 * j + lane;
-          okg[j] = sg[j] < M;
-#pragma unroll
-          for (int d = 0; d < 3; ++d) xg[j][d] = d < DIM ? xr[j][d] : (T)0;
-          cg[j] = okg[j] ? sseg[sg[j]] : 0;
-          vg[j][0] = okg[j] ? svx[sg[j]] : (T)0;
-          vg[j][1] = okg[j] ? svy[sg[j]] : (T)0;
-          vg[j][2] = okg[j] ? svz[sg[j]] : (T)0;
-          dtg[j] = ct->dt[cg[j]];
-        }
-#pragma unroll
-        for (int d = 0; d < DIM; ++d)
-#pragma unroll
-          for (int k = 0; k + W < R; ++k) xr[k][d] = xr[k + W][d];
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-          const InstParams& Pj = inst_params<ONE>(a, ct->inst[cg[j]]);
-          fg[j] = flight_fast<T, DIM>(Pj, xg[j], vg[j], dtg[j]);
-          kg[j] = (uint32_t)Pj.cell_off + cell_of<T, DIM>(Pj, xg[j]);
-        }
-#pragma unroll 1
-        for (int j = 0; j < W; ++j) {
-          uint32_t key = kSentinel;
-          if (okg[0]) {
-            key = kg[0];
-            if (!fg[0]) {
-              const int c = cg[0];
-              const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-              const bool gone = move_particle<T, DIM>(P, a.surf, xg[0], vg[0], dtg[0], step, kPurpWall,
-                                                      (uint32_t)ct->kl[c], (uint32_t)(sg[0] - ct->off[c]), 0u, a.err);
-              key = gone ? kSentinel : (uint32_t)P.cell_off + cell_of<T, DIM>(P, xg[0]);
-            }
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) Bx[d][p0 + sg[0]] = xg[0][d];
-            Bv[0][p0 + sg[0]] = vg[0][0];
-            Bv[1][p0 + sg[0]] = vg[0][1];
-            Bv[2][p0 + sg[0]] = vg[0][2];
-            a.key[p0 + sg[0]] = key;
-          }
-          warp_count(key, a.count);
-#pragma unroll
-          for (int i = 0; i + 1 < W; ++i) {
-            sg[i] = sg[i + 1]; cg[i] = cg[i + 1]; okg[i] = okg[i + 1]; fg[i] = fg[i + 1];
-            dtg[i] = dtg[i + 1]; kg[i] = kg[i + 1];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-              xg[i][d] = xg[i + 1][d];
-              vg[i][d] = vg[i + 1][d];
-            }
-          }
-        }
-      }
-    } else {
-#pragma unroll 1
-    for (int u = 0; u < R; ++u) {
-      const int sb = sb0 + 32 * u;
-      if (sb >= M) break;
-      const int s = sb + lane;
-      uint32_t key = kSentinel;
-      T x[3] = {0, 0, 0};
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        x[d] = xr[0][d];
-#pragma unroll
-        for (int k = 0; k < R - 1; ++k) xr[k][d] = xr[k + 1][d];
-      }
-      if (s < M) {
-        const int c = sseg[s];
-        const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-        T v[3] = {svx[s], svy[s], svz[s]};
-        const bool gone = move_particle<T, DIM>(P, a.surf, x, v, ct->dt[c], step, kPurpWall,
-                                                (uint32_t)ct->kl[c], (uint32_t)(s - ct->off[c]), 0u, a.err);
-        if (!gone) key = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) Bx[d][p0 + s] = x[d];
-        Bv[0][p0 + s] = v[0];
-        Bv[1][p0 + s] = v[1];
-        Bv[2][p0 + s] = v[2];
-        a.key[p0 + s] = key;
-      }
-      warp_count(key, a.count);
-    }
-    }
+  // ---- 9. the post-collision velocities in the current cell order, for the
+  // free flight (k_flight)
+  T* Bv0 = (T*)a.Bvel[0] + p0;
+  T* Bv1 = (T*)a.Bvel[1] + p0;
+  T* Bv2 = (T*)a.Bvel[2] + p0;
+#pragma unroll 4
+  for (int s = lane; s < M; s += 32) {
+    Bv0[s] = svx[s];
+    Bv1[s] = svy[s];
+    Bv2[s] = svz[s];
   }
   __syncwarp();
 }
 
-template <class T, class A, int DIM, bool ONE, bool MESH = false>
+template <class T, class A, int DIM, bool ONE>
 __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, 1) k_collide(StepArgs a, int big) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2427,7 +2260,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, 1) k_collide(StepArgs 
       if ((int)(a.start[k0 + 1] - a.start[k0]) > kHugeCell) continue;  // k_collide_huge's cell
     }
     const long long t0 = clock64();
-    process_batch<T, A, DIM, ONE, MESH>(a, k0, G, ct, sidx, stag, sseg, svx, svy, svz);
+    process_batch<T, A, DIM, ONE>(a, k0, G, ct, sidx, stag, sseg, svx, svy, svz);
     if (!big) {
       // the batch's cost steers the next step's plan (no effect on results):
       // its cycles per particle in units of cyc[2] (1/16 of the last step's
@@ -2543,7 +2376,7 @@ __device__ __forceinline__ void block_sums(TabT* tb, int n, typename Acc::result
   __syncthreads();
 }
 
-template <class T, class A, int DIM, bool ONE, bool MESH = false>
+template <class T, class A, int DIM, bool ONE>
 __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
   using Acc = CellAcc<T, A>;
   constexpr bool kMixed = mixed_prec<T, A>();
@@ -2604,7 +2437,10 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
         so[0] = 0;
       }
       __syncthreads();
-      for (int s = tid; s < N; s += kHugeThreads) sidx[s] = ((const uint32_t*)svy)[s];
+      for (int s = tid; s < N; s += kHugeThreads) {
+        sidx[s] = ((const uint32_t*)svy)[s];
+        a.perm[p0 + s] = sidx[s];  // (for the free flight)
+      }
       __syncthreads();
     }
     // ---- 2. gather
@@ -2972,43 +2808,107 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
       a.rec[2 * NC + k] = tb->nres;
       a.rec[3 * NC + k] = tb->nar;
     }
-    // ---- 9. free flight of the next interval, key and histogram (every
-    // thread reads its slot's source index and velocity before it writes
-    // the slot's key, position and velocity)
-    {
-      T* Bx[3] = {(T*)a.Bpos[0], (T*)a.Bpos[1], (T*)a.Bpos[2]};
-      T* Bv[3] = {(T*)a.Bvel[0], (T*)a.Bvel[1], (T*)a.Bvel[2]};
-      const T dt = tb->dt;
-      __syncthreads();  // the clash tags (in the first B position array) are dead
-      for (int sb = 0; sb < N; sb += kHugeThreads) {
-        const int s = sb + tid;
-        uint32_t key = kSentinel;
-        if (s < N) {
-          const uint32_t o = sidx[s];
-          T x[3] = {0, 0, 0};
+    // ---- 9. the post-collision velocities, for the free flight
+    if (N <= huge_smem_cap<T>())
+      for (int s = tid; s < N; s += kHugeThreads) {
+        ((T*)a.Bvel[0])[p0 + s] = svx[s];
+        ((T*)a.Bvel[1])[p0 + s] = svy[s];
+        ((T*)a.Bvel[2])[p0 + s] = svz[s];
+      }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Free flight of the next interval (Step 2), new key and histogram: one
+// thread per slot of the current cell order, kFlightPer slots per thread
+// (strided by the block) whose loads are in flight together.  Its inputs are
+// the source index and the post-collision velocity of the slot (coalesced)
+// and the source's position (runs of neighbouring indices).  The slot's cell
+// -- for the instance, the wall draws' counters and the O-grid's walk -- is
+// the source's key of the last step.
+// ---------------------------------------------------------------------------
+constexpr int kFlightThreads = 256;
+template <class T>
+constexpr int kFlightPer = sizeof(T) == 4 ? 2 : 1;
+
+template <class T, int DIM, bool ONE, bool MESH>
+__global__ void __launch_bounds__(kFlightThreads, sizeof(T) == 4 ? 4 : 3) k_flight(StepArgs a) {
+  constexpr int R = kFlightPer<T>;
+  const int64_t M = (int64_t)a.start[a.NC];
+  const uint32_t step = *a.step;
+  constexpr int64_t tile = (int64_t)kFlightThreads * R;
+  const T dt0 = ONE ? (T)a.dt_cur[0] : (T)0;
+  for (int64_t b0 = (int64_t)blockIdx.x * tile; b0 < M; b0 += (int64_t)gridDim.x * tile) {
+    uint32_t og[R], cg[R];
+    T xg[R][3], vg[R][3];
 #pragma unroll
-          for (int d = 0; d < DIM; ++d) x[d] = ((const T*)a.Apos[d])[o];
-          T v[3] = {svx[s], svy[s], svz[s]};
-          if constexpr (MESH) {
-            int64_t kn = kl;
-            const bool gone = mesh_walk<T>(Pi, (const T*)a.mface, a.surf, kn, x, v, dt, step, kPurpWall, kl,
-                                           (uint32_t)s, 0u, a.err, false);
-            if (!gone) key = (uint32_t)(Pi.cell_off + kn);
-          } else {
-            const bool gone = move_particle<T, DIM>(Pi, a.surf, x, v, dt, step, kPurpWall, kl, (uint32_t)s, 0u, a.err);
-            if (!gone) key = (uint32_t)Pi.cell_off + cell_of<T, DIM>(Pi, x);
-          }
+    for (int j = 0; j < R; ++j) {
+      const int64_t s = b0 + (int64_t)j * kFlightThreads + threadIdx.x;
+      og[j] = s < M ? a.perm[s] : kSentinel;
 #pragma unroll
-          for (int d = 0; d < DIM; ++d) Bx[d][p0 + s] = x[d];
-          Bv[0][p0 + s] = v[0];
-          Bv[1][p0 + s] = v[1];
-          Bv[2][p0 + s] = v[2];
-          a.key[p0 + s] = key;
-        }
-        warp_count(key, a.count);
+      for (int d = 0; d < 3; ++d) {
+        xg[j][d] = 0;
+        vg[j][d] = s < M ? ((const T*)a.Bvel[d])[s] : (T)0;
       }
     }
-    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      cg[j] = 0;
+      if (og[j] != kSentinel) {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) xg[j][d] = ((const T*)a.Apos[d])[og[j]];
+        if (MESH || !ONE) cg[j] = a.key_in[og[j]];
+      }
+    }
+#pragma unroll 1
+    for (int j = 0; j < R; ++j) {
+      const int64_t s = b0 + (int64_t)j * kFlightThreads + threadIdx.x;
+      uint32_t key = kSentinel;
+      if (s < M) {
+        T* x = xg[0];
+        T* v = vg[0];
+        const uint32_t inst = ONE ? 0u : a.cell_inst[cg[0]];
+        const InstParams& P = inst_params<ONE>(a, inst);
+        const T dt = ONE ? dt0 : (T)a.dt_cur[inst];
+        bool hit = false;  // the velocity changed (a wall event)
+        if constexpr (MESH) {
+          const int64_t k0 = (int64_t)cg[0] - P.cell_off;
+          int64_t kl = k0;
+          const bool gone = mesh_walk<T>(P, (const T*)a.mface, a.surf, kl, x, v, dt, step, kPurpWall, (uint32_t)k0,
+                                         (uint32_t)(s - a.start[cg[0]]), 0u, a.err, false);
+          hit = true;
+          if (!gone) key = (uint32_t)(P.cell_off + kl);
+        } else {
+          bool gone = false;
+          if (!flight_fast<T, DIM>(P, x, v, dt)) {
+            const uint32_t c = ONE ? a.key_in[og[0]] : cg[0];
+            gone = move_particle<T, DIM>(P, a.surf, x, v, dt, step, kPurpWall, (uint32_t)(c - P.cell_off),
+                                         (uint32_t)(s - a.start[c]), 0u, a.err);
+            hit = true;
+          }
+          if (!gone) key = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
+        }
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) ((T*)a.Bpos[d])[s] = x[d];
+        if (hit) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) ((T*)a.Bvel[d])[s] = v[d];
+        }
+        a.key[s] = key;
+      }
+      warp_count(key, a.count);
+#pragma unroll
+      for (int i = 0; i + 1 < R; ++i) {
+        og[i] = og[i + 1];
+        cg[i] = cg[i + 1];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          xg[i][d] = xg[i + 1][d];
+          vg[i][d] = vg[i + 1][d];
+        }
+      }
+    }
   }
 }
 

@@ -119,6 +119,7 @@ struct StepArgs {
   const void* Avel[3];
   void* Bpos[3];
   void* Bvel[3];
+  const uint32_t* key_in;  // [cap]  key (cell) of each A source
   uint32_t* key;        // [cap]   key of each B slot
   uint32_t* perm;       // [cap]   slot -> source index in A (sub-cells, FP32: re-ordered in place)
   const uint32_t* start;// [NC+1]  cell offsets of the current state
@@ -192,7 +193,8 @@ struct KernelSet {
   void (*collide)(int dim, const StepArgs& a, bool big, int grid, int warps, cudaStream_t s);
   void (*collide_huge)(int dim, const StepArgs& a, int grid, cudaStream_t s);
   size_t (*collide_smem)(int warps, int cap);
-  int (*collide_blocks_per_sm)(int dim, int warps, int cap, bool one, bool mesh);
+  void (*flight)(int dim, const StepArgs& a, int nsm, cudaStream_t s);
+  int (*collide_blocks_per_sm)(int dim, int warps, int cap, bool one);
   cudaError_t (*configure)();
   void (*inject)(int dim, const InjectArgs& a, int pass, cudaStream_t s);
   void (*moments)(const StepArgs& a, int64_t c0, int64_t c1, double* out, cudaStream_t s);

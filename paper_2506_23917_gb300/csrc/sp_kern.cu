@@ -17,45 +17,59 @@ namespace {
 using T = SP_KT;
 using A = SP_KA;
 
-template <int DIM, bool ONE, bool MESH>
+template <int DIM, bool ONE>
 void collide_dim1(const StepArgs& a, bool big, int grid, int warps, cudaStream_t s) {
   if (!big) {
     const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(a.cap_small);
-    k_collide<T, A, DIM, ONE, MESH><<<grid, 32 * warps, smem, s>>>(a, 0);
+    k_collide<T, A, DIM, ONE><<<grid, 32 * warps, smem, s>>>(a, 0);
   } else {
     const size_t smem = warp_stage_bytes<T, A>(a.big_cap);
-    k_collide<T, A, DIM, ONE, MESH><<<grid, 32, smem, s>>>(a, 1);
+    k_collide<T, A, DIM, ONE><<<grid, 32, smem, s>>>(a, 1);
   }
 }
 
-template <int DIM, bool MESH = false>
+template <int DIM>
 void collide_dim(const StepArgs& a, bool big, int grid, int warps, cudaStream_t s) {
-  if (a.one) collide_dim1<DIM, true, MESH>(a, big, grid, warps, s);
-  else collide_dim1<DIM, false, MESH>(a, big, grid, warps, s);
+  if (a.one) collide_dim1<DIM, true>(a, big, grid, warps, s);
+  else collide_dim1<DIM, false>(a, big, grid, warps, s);
 }
 
-// (O-grid instances are 2-D: their kernels take the face-crossing flight)
 void collide(int dim, const StepArgs& a, bool big, int grid, int warps, cudaStream_t s) {
   if (dim == 1) collide_dim<1>(a, big, grid, warps, s);
-  else if (dim == 2 && a.mesh) collide_dim<2, true>(a, big, grid, warps, s);
   else if (dim == 2) collide_dim<2>(a, big, grid, warps, s);
   else collide_dim<3>(a, big, grid, warps, s);
 }
 
 size_t collide_smem(int warps, int cap) { return (size_t)warps * warp_stage_bytes<T, A>(cap); }
 
-template <int DIM, bool MESH = false>
+template <int DIM>
 void collide_huge_dim(const StepArgs& a, int grid, cudaStream_t s) {
   const size_t smem = huge_smem_bytes<T, A>();
-  if (a.one) k_collide_huge<T, A, DIM, true, MESH><<<grid, kHugeThreads, smem, s>>>(a);
-  else k_collide_huge<T, A, DIM, false, MESH><<<grid, kHugeThreads, smem, s>>>(a);
+  if (a.one) k_collide_huge<T, A, DIM, true><<<grid, kHugeThreads, smem, s>>>(a);
+  else k_collide_huge<T, A, DIM, false><<<grid, kHugeThreads, smem, s>>>(a);
 }
 
 void collide_huge(int dim, const StepArgs& a, int grid, cudaStream_t s) {
   if (dim == 1) collide_huge_dim<1>(a, grid, s);
-  else if (dim == 2 && a.mesh) collide_huge_dim<2, true>(a, grid, s);
   else if (dim == 2) collide_huge_dim<2>(a, grid, s);
   else collide_huge_dim<3>(a, grid, s);
+}
+
+template <int DIM, bool MESH = false>
+void flight_dim(const StepArgs& a, int grid, cudaStream_t s) {
+  if (a.one) k_flight<T, DIM, true, MESH><<<grid, kFlightThreads, 0, s>>>(a);
+  else k_flight<T, DIM, false, MESH><<<grid, kFlightThreads, 0, s>>>(a);
+}
+
+// (O-grid instances are 2-D: their kernels take the face-crossing flight)
+void flight(int dim, const StepArgs& a, int nsm, cudaStream_t s) {
+  const int64_t tile = (int64_t)kFlightThreads * kFlightPer<T>;
+  const int64_t need = (a.cap + tile - 1) / tile, most = (int64_t)nsm * 8;
+  const int g = (int)(need < most ? need : most);
+  if (dim == 1) flight_dim<1>(a, g, s);
+  else if (dim == 2 && a.mesh) flight_dim<2, true>(a, g, s);
+  else if (dim == 2) flight_dim<2>(a, g, s);
+  else flight_dim<3>(a, g, s);
 }
 
 template <int DIM>
@@ -128,58 +142,54 @@ void stage_in(int dim, const S* pos, const S* vel, int64_t n, void* const dpos[3
                                             (T*)dvel[0], (T*)dvel[1], (T*)dvel[2], off, part_inst, inst);
 }
 
-template <int DIM, bool ONE, bool MESH>
+template <int DIM, bool ONE>
 cudaError_t configure_dim1() {
-  cudaError_t e = cudaFuncSetAttribute(k_collide<T, A, DIM, ONE, MESH>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_collide<T, A, DIM, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kMaxDynSmem);
   if (e == cudaSuccess)  // staging lives in shared memory: prefer the largest carveout
-    e = cudaFuncSetAttribute(k_collide<T, A, DIM, ONE, MESH>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
+    e = cudaFuncSetAttribute(k_collide<T, A, DIM, ONE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_collide_huge<T, A, DIM, ONE, MESH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_collide_huge<T, A, DIM, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)huge_smem_bytes<T, A>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_collide_huge<T, A, DIM, ONE, MESH>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    e = cudaFuncSetAttribute(k_collide_huge<T, A, DIM, ONE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
-template <int DIM, bool MESH = false>
+template <int DIM>
 cudaError_t configure_dim() {
-  cudaError_t e = configure_dim1<DIM, true, MESH>();
-  if (e == cudaSuccess) e = configure_dim1<DIM, false, MESH>();
+  cudaError_t e = configure_dim1<DIM, true>();
+  if (e == cudaSuccess) e = configure_dim1<DIM, false>();
   return e;
 }
 
 cudaError_t configure() {
   cudaError_t e = configure_dim<1>();
   if (e == cudaSuccess) e = configure_dim<2>();
-  if (e == cudaSuccess) e = configure_dim<2, true>();
   if (e == cudaSuccess) e = configure_dim<3>();
   return e;
 }
 
-template <int DIM, bool MESH = false>
+template <int DIM>
 int blocks_per_sm_dim(int warps, size_t smem, bool one) {
   int n = 0;
   if (one)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide<T, A, DIM, true, MESH>, 32 * warps, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide<T, A, DIM, true>, 32 * warps, smem);
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide<T, A, DIM, false, MESH>, 32 * warps, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_collide<T, A, DIM, false>, 32 * warps, smem);
   return n;
 }
 
-int blocks_per_sm(int dim, int warps, int cap, bool one, bool mesh) {
+int blocks_per_sm(int dim, int warps, int cap, bool one) {
   const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(cap);
   if (dim == 1) return blocks_per_sm_dim<1>(warps, smem, one);
-  if (dim == 2 && mesh) return blocks_per_sm_dim<2, true>(warps, smem, one);
   if (dim == 2) return blocks_per_sm_dim<2>(warps, smem, one);
   return blocks_per_sm_dim<3>(warps, smem, one);
 }
 }  // namespace
 
 const KernelSet& SP_CAT(kernels, SP_TAG)() {
-  static const KernelSet k = {collide,  collide_huge, collide_smem,     blocks_per_sm,   configure,
+  static const KernelSet k = {collide,  collide_huge, collide_smem, flight, blocks_per_sm, configure,
                               inject,   moments,      keys,             keys_mesh,       gather,
                               stage_in<double>,       stage_in<float>};
   return k;
