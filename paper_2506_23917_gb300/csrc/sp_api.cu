@@ -72,6 +72,7 @@ struct sp_ctx {
   unsigned long long* dt_min = nullptr;
   uint32_t *step_d = nullptr, *Mcur = nullptr, *Mtot = nullptr;
   unsigned long long* err = nullptr;
+  unsigned long long* herr = nullptr;  // page-locked copy of err (check_errors)
   GhostCell* ghosts = nullptr;
   int64_t n_ghost = 0;
   uint32_t *gcount = nullptr, *goff = nullptr, *gscan_part = nullptr;
@@ -641,9 +642,11 @@ sp_status build_graphs(sp_ctx* c) {
   return SP_OK;
 }
 
+// Waits for the context's stream and looks at its error counters (copied to
+// page-locked memory behind the work in flight: one wait for both).
 sp_status check_errors(sp_ctx* c) {
-  unsigned long long h[kNumErr];
-  CK(cudaMemcpyAsync(h, c->err, sizeof h, cudaMemcpyDeviceToHost, c->stream));
+  unsigned long long* h = c->herr;
+  CK(cudaMemcpyAsync(h, c->err, 8 * kNumErr, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   if (h[kErrCapacity] || h[kErrCellCap]) return SP_ERR_CAPACITY;
   return SP_OK;
@@ -857,6 +860,7 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
     CK(dalloc(&c->Mcur, 4));
     CK(dalloc(&c->Mtot, 4));
     CK(dalloc(&c->err, 8 * kNumErr));
+    CK(cudaHostAlloc((void**)&c->herr, 8 * kNumErr, cudaHostAllocDefault));
     CK(dalloc(&c->ghosts, sizeof(GhostCell) * std::max<int64_t>(c->n_ghost, 1)));
     CK(dalloc(&c->gcount, 4 * std::max<int64_t>(c->n_ghost, 1)));
     CK(dalloc(&c->goff, 4 * (std::max<int64_t>(c->n_ghost, 1) + 1)));
@@ -1171,22 +1175,17 @@ sp_status sp_moments(sp_ctx* c, int inst, int kind, double* out, int n_fields) {
   const InstParams& P = c->hP[inst];
   const int64_t nc = P.ncells;
   const int nf = std::min(n_fields, (int)SP_NFIELDS);
-  if (kind == 0) {
-    // page-locked host memory the device can address: the fields kernel
-    // writes its rows straight into it (the link transfer overlaps the
-    // FP64 work); otherwise a device buffer and one copy
-    cudaPointerAttributes pa;
-    double* direct = nullptr;
-    if (nf == SP_NFIELDS && cudaPointerGetAttributes(&pa, out) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
-        pa.devicePointer)
-      direct = (double*)pa.devicePointer;
-    cudaGetLastError();  // (a pointer unknown to CUDA leaves an error to clear)
-    if (direct) {
-      StepArgs a = make_step_args(c, c->cur);
-      c->K->moments(a, P.cell_off, P.cell_off + nc, direct, c->stream);
-      CK(cudaStreamSynchronize(c->stream));
-      return check_errors(c);
-    }
+  // page-locked host memory the device can address: the fields kernel
+  // writes its rows straight into it (the link transfer overlaps the
+  // FP64 work); otherwise a device buffer and one copy
+  cudaPointerAttributes pa;
+  double* d = nullptr;
+  if (nf == SP_NFIELDS && cudaPointerGetAttributes(&pa, out) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
+      pa.devicePointer)
+    d = (double*)pa.devicePointer;
+  cudaGetLastError();  // (a pointer unknown to CUDA leaves an error to clear)
+  const bool direct = d != nullptr;
+  if (!direct) {
     if (nc > c->mom_cells) {  // one device buffer, grown on demand
       CK(cudaStreamSynchronize(c->stream));
       if (c->mom) CK(cudaFree(c->mom));
@@ -1195,43 +1194,18 @@ sp_status sp_moments(sp_ctx* c, int inst, int kind, double* out, int n_fields) {
       CK(dalloc(&c->mom, 8 * SP_NFIELDS * nc));
       c->mom_cells = nc;
     }
-    double* d = c->mom;
+    d = c->mom;
+  }
+  if (kind == 0) {
     // (reproducible runs: every step leaves the cells in source order, so
     // each cell is summed in that order)
-    StepArgs a = make_step_args(c, c->cur);
+    const StepArgs a = make_step_args(c, c->cur);
     c->K->moments(a, P.cell_off, P.cell_off + nc, d, c->stream);
-    CK(cudaMemcpyAsync(out, d, 8 * nf * nc, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
   } else {
-    std::vector<double> S(8 * nc), vol(nc);
-    for (int f = 0; f < 8; ++f)
-      CK(cudaMemcpyAsync(S.data() + f * nc, c->samp + f * c->NC + P.cell_off, 8 * nc, cudaMemcpyDeviceToHost,
-                         c->stream));
-    CK(cudaMemcpyAsync(vol.data(), c->vol + P.cell_off, 8 * nc, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
     const int64_t nsamp = std::max<int64_t>(0, c->step_host - (int64_t)P.n_steady);
-    for (int64_t k = 0; k < nc; ++k) {
-      double f[SP_NFIELDS] = {0};
-      const double sN = S[k];
-      if (nsamp > 0) {
-        f[SP_F_N] = sN / (double)nsamp;
-        f[SP_F_n] = vol[k] > 0 ? f[SP_F_N] * P.Fn / vol[k] : 0.0;
-        f[SP_F_ratio] = S[7 * nc + k] / (double)nsamp;
-      }
-      if (sN > 0) {
-        double U[3], e = 0;
-        for (int d = 0; d < 3; ++d) {
-          U[d] = S[(1 + d) * nc + k] / sN;
-          e += S[(4 + d) * nc + k] / sN - U[d] * U[d];
-        }
-        f[SP_F_ux] = U[0];
-        f[SP_F_uy] = U[1];
-        f[SP_F_uz] = U[2];
-        f[SP_F_T] = e / (3.0 * P.R);
-      }
-      for (int i = 0; i < nf; ++i) out[(int64_t)i * nc + k] = f[i];
-    }
+    launch_mean_fields(c->samp, c->NC, c->vol, P.cell_off, nc, (double)nsamp, P.Fn, P.R, d, c->stream);
   }
+  if (!direct) CK(cudaMemcpyAsync(out, d, 8 * nf * nc, cudaMemcpyDeviceToHost, c->stream));
   return check_errors(c);
 }
 
@@ -1463,6 +1437,7 @@ sp_status sp_free(sp_ctx* c) {
                   c->big_count, c->vol, c->smax, c->rem, c->samp, c->rec, c->resamp, c->dP, c->dt_cur, c->dt_min,
                   c->step_d, c->Mcur, c->Mtot, c->err, c->ghosts, c->gcount, c->goff, c->gscan_part};
   for (void* p : ptrs) cudaFree(p);
+  if (c->herr) cudaFreeHost(c->herr);
   delete c;
   return SP_OK;
 }

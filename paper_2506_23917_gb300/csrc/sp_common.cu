@@ -3,6 +3,7 @@
 // writes the slot -> source permutation, and the end-of-step bookkeeping.
 #include <cstdint>
 
+#include "../../include/sp.h"
 #include "sp_internal.h"
 
 namespace sp {
@@ -257,7 +258,53 @@ __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, i
   }
 }
 
+// Time-averaged fields of nc cells (Step 6) from the Step 5 sums, as IEEE
+// operations without contraction.  Bound by the host link where out is
+// mapped host memory (96 B written per cell against 72 read).
+__global__ void k_mean_fields(const double* samp, int64_t NC, const double* vol, int64_t c0, int64_t nc, double nsamp,
+                              double Fn, double R3, double* out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nc) return;
+  double S[8];
+#pragma unroll
+  for (int f = 0; f < 8; ++f) S[f] = samp[f * NC + c0 + i];
+  const double V = vol[c0 + i], sN = S[0];
+  double n = 0, N = 0, ratio = 0, U[3] = {0, 0, 0}, T = 0;
+  if (nsamp > 0) {
+    N = sN / nsamp;
+    n = V > 0 ? __dmul_rn(N, Fn) / V : 0.0;
+    ratio = S[7] / nsamp;
+  }
+  if (sN > 0) {
+    double e = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      U[d] = S[1 + d] / sN;
+      e = __dadd_rn(e, __dsub_rn(S[4 + d] / sN, __dmul_rn(U[d], U[d])));
+    }
+    T = e / R3;
+  }
+  out[SP_F_N * nc + i] = N;
+  out[SP_F_n * nc + i] = n;
+  out[SP_F_ux * nc + i] = U[0];
+  out[SP_F_uy * nc + i] = U[1];
+  out[SP_F_uz * nc + i] = U[2];
+  out[SP_F_T * nc + i] = T;
+  out[SP_F_qx * nc + i] = 0;
+  out[SP_F_qy * nc + i] = 0;
+  out[SP_F_qz * nc + i] = 0;
+  out[SP_F_tau * nc + i] = 0;
+  out[SP_F_dtc * nc + i] = 0;
+  out[SP_F_ratio * nc + i] = ratio;
+}
+
 }  // namespace
+
+void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64_t c0, int64_t nc, double nsamp,
+                        double Fn, double R, double* out, cudaStream_t s) {
+  if (nc <= 0) return;
+  k_mean_fields<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(samp, NC, vol, c0, nc, nsamp, Fn, 3.0 * R, out);
+}
 
 void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int split, uint2* batches,
                  uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
