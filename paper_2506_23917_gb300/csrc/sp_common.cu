@@ -173,9 +173,15 @@ __global__ void k_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
 // rejections, or with many collision candidates, cost several times the
 // mean per particle, and a warp takes only a few batches per launch.
 // Class k's list is batches[k NC ...].  Batches are independent: their
-// order changes no result.
-__global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int split, uint2* batches,
-                       uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count) {
+// order changes no result.  A state too small to give every resident warp
+// of the collision launch (nwarps) a full batch is cut into smaller ones,
+// down to one cell each: the launch then lasts as long as one batch, whose
+// time is proportional to its particles (kPlanWaves batches per warp).
+constexpr int kPlanWaves = 1;
+__global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap_max, int nwarps, int split,
+                       uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count) {
+  const int64_t share = ((int64_t)start[NC] + (int64_t)nwarps * kPlanWaves - 1) / ((int64_t)nwarps * kPlanWaves);
+  const int cap = share < 32 ? 32 : share < cap_max ? (int)share : cap_max;
   // per block: the batches of each class (shared atomics), then one global
   // atomic per class for the block's place in the class list
   __shared__ uint32_t cnt[kBatchClasses], base[kBatchClasses];
@@ -216,7 +222,8 @@ __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, i
       while (kk < nc) {
         const int64_t before = kk > 0 ? __shfl_sync(0xFFFFFFFFu, cum, kk - 1) : 0;
         const int lbefore = kk > 0 ? __shfl_sync(0xFFFFFFFFu, lcum, kk - 1) : 0;
-        const unsigned fit = __ballot_sync(0xFFFFFFFFu, lane >= kk && lane < nc && cum - before <= cap &&
+        const unsigned fit = __ballot_sync(0xFFFFFFFFu, lane >= kk && lane < nc &&
+                                                          cum - before <= (lane == kk ? cap_max : cap) &&
                                                           lcum - lbefore <= 32);
         const int G = __popc(fit);
         if (G == 0) {  // the cell alone exceeds the staging area: big-cell list
@@ -306,13 +313,13 @@ void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64
   k_mean_fields<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(samp, NC, vol, c0, nc, nsamp, Fn, 3.0 * R, out);
 }
 
-void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int split, uint2* batches,
-                 uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
+void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int nwarps, int split,
+                 uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
   const int64_t chunks = (NC + 31) / 32;
   int64_t g = (chunks + 7) / 8;
   if (g > 4096) g = 4096;
   if (g < 1) g = 1;
-  k_plan<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, split, batches, nbatch, big_list, big_count);
+  k_plan<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, nwarps, split, batches, nbatch, big_list, big_count);
 }
 
 int64_t scan_partial_size(int64_t n) { return (n + kTile - 1) / kTile + 1; }
