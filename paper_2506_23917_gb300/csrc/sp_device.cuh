@@ -39,10 +39,27 @@ __device__ __forceinline__ uint4 philox10(uint32_t c0, uint32_t c1, uint32_t c2,
   return make_uint4(c0, c1, c2, c3);
 }
 
-// FP64 uniform in (0,1): 52 bits from two words, (2k+1) 2^-53.
+// FP64 uniform in (0,1): 52 bits from two words, (2k+1) 2^-53.  Formed as
+// (1 + k 2^-52) - (1 - 2^-53), exact in one subtraction: on GB300 an FP64
+// operation or 64-bit conversion holds the SM's FP64 pipe for ~17 cycles.
 __device__ __forceinline__ double u01d(uint32_t a, uint32_t b) {
   const unsigned long long k = ((unsigned long long)(a >> 6) << 26) | (unsigned long long)(b >> 6);
-  return (double)(2ull * k + 1ull) * 1.1102230246251565404236316680908203125e-16;
+  return __longlong_as_double((long long)(0x3FF0000000000000ull | k)) -
+         __longlong_as_double(0x3FEFFFFFFFFFFFFFll);
+}
+// The same uniform in FP32, to 2^-22 relative.
+__device__ __forceinline__ float u01d_approx(uint32_t a, uint32_t b) {
+  return fmaf((float)(a >> 6), 1.490116119384765625e-8f, (float)(2u * (b >> 6) + 1u) * 1.1102230246251565e-16f);
+}
+// An FP64 value in FP32 (truncated, relative error below 2^-23) by integer
+// operations only; zero below FP32's normal range, infinity above it.
+__device__ __forceinline__ float approx_f32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t e = (hi >> 20) & 0x7FFu;
+  uint32_t m = (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29);
+  if (e < 897u) m = 0u;
+  if (e > 1150u) m = 0x7F800000u;
+  return __uint_as_float(m | (hi & 0x80000000u));
 }
 // FP32 uniform in (0,1): 23 bits from one word, (2k+1) 2^-24.
 __device__ __forceinline__ float u01f(uint32_t a) {
@@ -164,32 +181,43 @@ __device__ __forceinline__ float tmax0(float x) { return fmaxf(x, 0.0f); }
 
 // cos / sin of 2 pi u
 __device__ __forceinline__ void sincos2pi(double u, double* s, double* c) {
-  const double th = 2.0 * kPi * u;
-  *s = sin(th);
-  *c = cos(th);
+  sincospi(2.0 * u, s, c);
 }
 __device__ __forceinline__ void sincos2pi(float u, float* s, float* c) { sincospif(2.0f * u, s, c); }
-__device__ __forceinline__ double cos2pi(double u) { return cos(2.0 * kPi * u); }
+__device__ __forceinline__ double cos2pi(double u) { return cospi(2.0 * u); }
 __device__ __forceinline__ float cos2pi(float u) { return cospif(2.0f * u); }
 
 // The five uniforms of NTC candidate kk: pair (u1, u2), acceptance u3,
 // scattering cos(chi) from u4 and azimuth from u5.  FP64 mode: three Philox
-// blocks (shared layout with the oracle).  FP32 mode: one block; u4 and u5
+// blocks (shared layout with the oracle), the third formed for accepted
+// candidates only.  FP32 mode: one block; u4 and u5
 // take 16 bits each of the fourth word ((2k+1) 2^-17), ample for angles.
 template <class T>
-struct NtcDraw {
-  T u1, u2, u3, u4, u5;
+struct NtcDraw;
+template <>
+struct NtcDraw<double> {
+  uint4 w0, w1;  // u1 u2, u3 u4
+  double u1, u2;
+  __device__ __forceinline__ double u3() const { return u01d(w1.x, w1.y); }
+  __device__ __forceinline__ float u3_approx() const { return u01d_approx(w1.x, w1.y); }
+  __device__ __forceinline__ double u4() const { return u01d(w1.z, w1.w); }
+};
+template <>
+struct NtcDraw<float> {
+  float u1, u2, u3, u4, u5;
 };
 __device__ __forceinline__ NtcDraw<double> ntc_draw(double, uint32_t step, uint32_t kl, uint32_t kk,
                                                     uint32_t key0, uint32_t key1) {
-  Uni<double> r(step, kl, kk, kPurpNtc << 24, key0, key1);
   NtcDraw<double> d;
-  d.u1 = r.get(0);
-  d.u2 = r.get(1);
-  d.u3 = r.get(2);
-  d.u4 = r.get(3);
-  d.u5 = r.get(4);
+  d.w0 = philox10(step, kl, kk, kPurpNtc << 24, key0, key1);
+  d.w1 = philox10(step, kl, kk, (kPurpNtc << 24) + 1u, key0, key1);
+  d.u1 = u01d(d.w0.x, d.w0.y);
+  d.u2 = u01d(d.w0.z, d.w0.w);
   return d;
+}
+__device__ __forceinline__ double ntc_u5(uint32_t step, uint32_t kl, uint32_t kk, uint32_t key0, uint32_t key1) {
+  const uint4 w = philox10(step, kl, kk, (kPurpNtc << 24) + 2u, key0, key1);
+  return u01d(w.x, w.y);
 }
 __device__ __forceinline__ NtcDraw<float> ntc_draw(float, uint32_t step, uint32_t kl, uint32_t kk,
                                                    uint32_t key0, uint32_t key1) {
@@ -201,6 +229,46 @@ __device__ __forceinline__ NtcDraw<float> ntc_draw(float, uint32_t step, uint32_
   d.u4 = (float)(2u * (w.w >> 16) + 1u) * 7.62939453125e-6f;
   d.u5 = (float)(2u * (w.w & 0xFFFFu) + 1u) * 7.62939453125e-6f;
   return d;
+}
+
+// FP64 mode's test of an NTC candidate: sigma c = coef c_r^ex costs a square
+// root and a power, over 100 operations of the FP64 pipe, and is needed only
+// for decisions -- whether it raises (sigma c)_max, and whether
+// u3 < sigma c / (sigma c)_max.  An FP32 estimate (relative error below 1e-5,
+// the sum of the rounding of its inputs, powf and ex ln c_r) settles both
+// unless it comes within 1e-4 of the line; only then is the FP64 value
+// formed, so that every decision is the FP64 one.
+struct NtcTest {
+  double sc;   // sigma c where it was formed, else -1 (then below S)
+  float est;   // estimate of sigma c / S, S = (sigma c)_max before the round
+  bool exact;  // sc was formed
+};
+__device__ __forceinline__ double ntc_sigc(double g0, double g1, double g2, double coef, double ex) {
+  return coef * cpow(csqrt(g0 * g0 + g1 * g1 + g2 * g2), ex);
+}
+__device__ __forceinline__ NtcTest ntc_test(double g0, double g1, double g2, double S, double coef, double ex,
+                                            float coef32, float ex32) {
+  NtcTest o;
+  const float x = approx_f32(g0), y = approx_f32(g1), z = approx_f32(g2), S32 = approx_f32(S);
+  const float c2 = x * x + y * y + z * z;
+  const float sc32 = coef32 * powf(sqrtf(c2), ex32);
+  o.est = sc32 / S32;
+  const bool sure = c2 > 1e-30f && c2 < 1e30f && S32 > 1e-30f && S32 < 1e30f && sc32 > 1e-30f && o.est < 0.9999f;
+  o.exact = !sure;
+  o.sc = -1.0;
+  if (!sure) o.sc = ntc_sigc(g0, g1, g2, coef, ex);
+  return o;
+}
+// u3 < sigma c / smL, with smL >= S the running maximum up to the candidate.
+__device__ __forceinline__ bool ntc_pass(const NtcTest& o, const NtcDraw<double>& dr, double g0, double g1, double g2,
+                                         double S, double smL, double coef, double ex) {
+  if (!o.exact && smL == S) {
+    const float u = dr.u3_approx();
+    if (u < o.est * 0.9999f) return true;
+    if (u > o.est * 1.0001f) return false;
+  }
+  const double sc = o.exact ? o.sc : ntc_sigc(g0, g1, g2, coef, ex);
+  return dr.u3() < sc / smL;
 }
 
 template <class T>
@@ -366,6 +434,70 @@ __device__ __forceinline__ bool flight_fast(const InstParams& P, T* x, const T* 
     for (int d = 0; d < DIM; ++d) x[d] = xe[d];
   }
   return ok;
+}
+
+// FP64 state: the same question asked in FP32 first, on truncated positions
+// and velocities (relative error below 2^-22; P.g32.eps is 1e-5 of the span,
+// the magnitude of the box's coordinates).  A particle that starts and ends
+// inside the box by that margin, and whose path keeps further from the
+// body's centre than r by 4e-6 of the lengths involved plus the rounding of
+// the coordinates, flies straight in FP64 too (there the margins are 1e10
+// roundings wide): 2 DIM operations of the FP64 pipe instead of about 45.
+template <int DIM>
+__device__ __forceinline__ bool flight_clear(const InstParams& P, const double* x, const double* v, double trem) {
+  const Geo<float>& G = P.g32;
+  const float dt = approx_f32(trem);
+  float xf[DIM], vf[DIM];
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    xf[d] = approx_f32(x[d]);
+    vf[d] = approx_f32(v[d]);
+    const float xe = fmaf(vf[d], dt, xf[d]);
+    ok = ok && xe > G.lo[d] + G.eps[d] && xe < G.hi[d] - G.eps[d] && fabsf(xf[d]) + fabsf(vf[d]) * dt < 2e5f * G.eps[d];
+  }
+  if (P.body != 0) {
+    float dx[DIM], bb = 0, aa = 0, dd = 0, m = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      if (d == 2 && P.body == 1) break;
+      dx[d] = xf[d] - G.body_c[d];
+      bb = fmaf(vf[d], dx[d], bb);
+      aa = fmaf(vf[d], vf[d], aa);
+      dd = fmaf(dx[d], dx[d], dd);
+      m += 0.05f * G.eps[d] + 4e-7f * fabsf(G.body_c[d]) + 4e-6f * (fabsf(dx[d]) + fabsf(vf[d]) * dt);
+    }
+    // the path's closest point (a clamped time; its own error counts only
+    // in second order)
+    const float ts = fminf(fmaxf(__fdividef(-bb, aa), 0.0f), dt);
+    float pp = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      if (d == 2 && P.body == 1) break;
+      const float p = fmaf(vf[d], ts, dx[d]);
+      pp = fmaf(p, p, pp);
+    }
+    const float rm = G.body_r + m;
+    ok = ok && aa > 1e-30f && aa < 1e30f && dd < 1e30f && pp > rm * rm * 1.00001f;
+  }
+  return ok;
+}
+// The cell of a point flight_clear has found inside the box: the FP32
+// coordinate decides unless it comes within 1e-6 of the span of a cell face.
+template <int DIM>
+__device__ __forceinline__ uint32_t cell_of_clear(const InstParams& P, const double* x) {
+  const Geo<float>& G = P.g32;
+  uint32_t idx[3] = {0, 0, 0};
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    const float u = (approx_f32(x[d]) - G.lo[d]) * G.inv_d[d], f = floorf(u);
+    const float mg = 0.1f * G.eps[d] * G.inv_d[d];
+    ok = ok && u - f > mg && u - f < 1.0f - mg && f >= 0.0f && f < (float)P.n[d];
+    idx[d] = (uint32_t)(int)f;
+  }
+  if (!ok) return cell_of<double, DIM>(P, x);
+  return idx[0] + (uint32_t)P.n[0] * (idx[1] + (uint32_t)P.n[1] * idx[2]);
 }
 
 // Wall tallies of one body hit while sampling (FP64 atomics): the momentum
@@ -1351,9 +1483,57 @@ __device__ __forceinline__ void cell_math(const StepArgs& a, const InstParams& P
 // modes: one Philox block per attempt (block 1 + t; block 0 holds the
 // Bernoulli draw), the two angles sharing a word, 16 bits each, and A formed
 // with the per-particle constants kA = (1 - Pr) / (5 (RT)^2), iRT = 1 / RT.
+// FP64 mode: an attempt costs some 250 operations of the FP64 pipe (two
+// logarithms, two square roots, three sines or cosines), and most attempts
+// are rejected.  In units of sqrt(RT), A = 1 + (kq . c)(|c|^2 - 5) with
+// kq = (1 - Pr) q_s / (5 (RT)^(3/2)): an FP32 evaluation, whose error stays
+// below 1e-5 |kq|_1 (1 + |c|_1)(|c|^2 + 5), rejects the attempts that are
+// beyond that margin; the others are evaluated in FP64, so that every
+// decision and every accepted velocity is the FP64 one.
+struct ShakhovFilter {
+  float kx, ky, kz, amax;  // amax < 0: no filter (values outside FP32's range)
+};
+__device__ __forceinline__ ShakhovFilter shakhov_filter(double RT, double Amax, double omp, double q0, double q1,
+                                                        double q2) {
+  ShakhovFilter f;
+  const float rt = approx_f32(RT), k = 0.2f * approx_f32(omp) / (rt * sqrtf(rt));
+  f.kx = k * approx_f32(q0);
+  f.ky = k * approx_f32(q1);
+  f.kz = k * approx_f32(q2);
+  f.amax = approx_f32(Amax);
+  const float big = fabsf(f.kx) + fabsf(f.ky) + fabsf(f.kz) + f.amax;
+  if (!(rt > 1e-20f && rt < 1e20f && big < 1e15f)) f.amax = -1.0f;
+  return f;
+}
+__device__ __forceinline__ ShakhovFilter shakhov_filter(float, float, float, float, float, float) { return {}; }
+// -ln(u) of the uniform with words (a, b), relative error of a few 1e-7 also
+// near u = 1
+__device__ __forceinline__ float neg_log_approx(uint32_t a, uint32_t b) {
+  if (a >> 31) {  // 1 - u = (2 k' + 1) 2^-53, k' the complement
+    const float d = u01d_approx(~a, ~b);
+    return -log1pf(-d);
+  }
+  return -logf(u01d_approx(a, b));
+}
+__device__ __forceinline__ bool shakhov_surely_rejected(const uint32_t* wa, const uint32_t* wb,
+                                                        const ShakhovFilter& f) {
+  if (!(f.amax > 0.0f)) return false;
+  const float r2 = sqrtf(2.0f * neg_log_approx(wa[1], wb[1])), r4 = sqrtf(2.0f * neg_log_approx(wa[3], wb[3]));
+  float sn, cs;
+  sincospif(2.0f * u01d_approx(wa[2], wb[2]), &sn, &cs);
+  const float c0 = r2 * cospif(2.0f * u01d_approx(wa[0], wb[0])), c1 = r4 * cs, c2 = r4 * sn;
+  const float cc = c0 * c0 + c1 * c1 + c2 * c2;
+  const float A = 1.0f + (f.kx * c0 + f.ky * c1 + f.kz * c2) * (cc - 5.0f);
+  const float err = 1e-5f * (fabsf(f.kx) + fabsf(f.ky) + fabsf(f.kz)) *
+                        (1.0f + fabsf(c0) + fabsf(c1) + fabsf(c2)) * (cc + 5.0f);
+  const float lim = u01d_approx(wa[4], wb[4]) * f.amax;
+  return lim * 0.99999f > A + err + 1e-5f;
+}
+
 template <class T>
 __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, T Amax, T omp, T RT, T kA, T iRT,
-                                                T q0, T q1, T q2, T* C0, T* C1, T* C2) {
+                                                T q0, T q1, T q2, const ShakhovFilter& fl, bool last, T* C0, T* C1,
+                                                T* C2) {
   T R1, R2, R3, R4, R5;
   if constexpr (sizeof(T) == 4) {
     const uint4 w = philox10(r.c0, r.c1, r.c2, r.c3 + 1u + (uint32_t)t, r.k0, r.k1);
@@ -1363,9 +1543,22 @@ __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, 
     R3 = (float)(2u * (w.z & 0xFFFFu) + 1u) * 7.62939453125e-6f;
     R5 = u01f(w.w);
   } else {
-    T Rt[5];
-    uni_run<T, 5>(r, 1 + 5 * t, Rt);
-    R1 = Rt[0]; R2 = Rt[1]; R3 = Rt[2]; R4 = Rt[3]; R5 = Rt[4];
+    // the words of the five uniforms: uniform q in half q & 1 of block q / 2
+    uint32_t wa[5], wb[5];
+    const int q0u = 1 + 5 * t;
+#pragma unroll 1
+    for (int b = q0u >> 1; b <= (q0u + 4) >> 1; ++b) {
+      const uint4 w = philox10(r.c0, r.c1, r.c2, r.c3 + (uint32_t)b, r.k0, r.k1);
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if ((q0u + j) >> 1 == b) {
+          wa[j] = (q0u + j) & 1 ? w.z : w.x;
+          wb[j] = (q0u + j) & 1 ? w.w : w.y;
+        }
+    }
+    if (!last && shakhov_surely_rejected(wa, wb, fl)) return false;  // (the last one is kept whatever it is)
+    R1 = u01d(wa[0], wb[0]); R2 = u01d(wa[1], wb[1]); R3 = u01d(wa[2], wb[2]);
+    R4 = u01d(wa[3], wb[3]); R5 = u01d(wa[4], wb[4]);
   }
   // (max: near R = 1 the approximate logarithm may round above 0)
   const T r2 = csqrt(tmax0(-clog(R2))), r4 = csqrt(tmax0(-clog(R4)));
@@ -1736,18 +1929,32 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
           const T ax = svx[ci], ay = svy[ci], az = svz[ci];
           const T bx = svx[cj], by = svy[cj], bz = svz[cj];
           const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
-          const T cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
-          const T sc = coef * cpow(cr, ex);
-          if (sc > smx) smx = sc;  // the inclusive running maximum
+          T cr, u4, u5;
           bool pass;
-          if constexpr (sizeof(T) == 4) pass = dr.u3 * smx < sc;
-          else pass = dr.u3 < sc / smx;
+          if constexpr (sizeof(T) == 4) {
+            cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+            const T sc = coef * cpow(cr, ex);
+            if (sc > smx) smx = sc;  // the inclusive running maximum
+            pass = dr.u3 * smx < sc;
+            u4 = dr.u4;
+            u5 = dr.u5;
+          } else {
+            const NtcTest tt = ntc_test(g0, g1, g2, smx, coef, ex, Pi.g32.sigc_coef, Pi.g32.sigc_exp);
+            const T S = smx;
+            if (tt.sc > smx) smx = tt.sc;
+            pass = ntc_pass(tt, dr, g0, g1, g2, S, smx, coef, ex);
+            if (pass) {
+              cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+              u4 = dr.u4();
+              u5 = ntc_u5(step, (uint32_t)ct->kl[lane], (uint32_t)k, Pi.key0, Pi.key1);
+            }
+          }
           if (pass) {
             ++nacc_l;
-            const T cchi = (T)2.0 * dr.u4 - (T)1.0;
+            const T cchi = (T)2.0 * u4 - (T)1.0;
             const T schi = csqrt((T)1.0 - cchi * cchi);
             T sn, cs;
-            sincos2pi(dr.u5, &sn, &cs);
+            sincos2pi(u5, &sn, &cs);
             const T w0 = cchi, w1 = schi * cs, w2 = schi * sn;
             const T q0 = ax + bx, q1 = ay + by, q2 = az + bz;
             svx[ci] = (T)0.5 * (q0 - cr * w0);
@@ -1771,7 +1978,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     const int g = base + lane;
     const bool valid = g < ctot;
     int c = 255, ci = 0, cj = 0;
-    T u3 = 0, u4 = 0, u5 = 0;
+    NtcDraw<T> dr = {};
     if (valid) {
       int lo = 0, hi = G - 1;  // largest cell index with coff <= g
       while (lo < hi) {
@@ -1781,16 +1988,16 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       c = lo;
       const int N = ct->off[c + 1] - ct->off[c];
       const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-      const NtcDraw<T> dr = ntc_draw((T)0, step, (uint32_t)ct->kl[c], (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
-      u3 = dr.u3;
-      u4 = dr.u4;
-      u5 = dr.u5;
+      dr = ntc_draw((T)0, step, (uint32_t)ct->kl[c], (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
       select_pair(N, dr.u1, dr.u2, ct->soff[c], P.nsub, &ci, &cj);
       ci += ct->off[c];
       cj += ct->off[c];
     }
-    const int cnext = __shfl_down_sync(kFull, c, 1);
+    const int cnext = __shfl_down_sync(kFull, c, 1), cprev = __shfl_up_sync(kFull, c, 1);
     const bool seg_last = valid && (lane == 31 || cnext != c);
+    // the first lane of this lane's cell
+    const unsigned upto = 0xFFFFFFFFu >> (31 - lane);
+    const int seg0 = 31 - __clz((int)(__ballot_sync(kFull, lane == 0 || c != cprev) & upto));
     const T coef = valid ? geo<T>(inst_params<ONE>(a, ct->inst[c])).sigc_coef : (T)0;
     const T ex = valid ? geo<T>(inst_params<ONE>(a, ct->inst[c])).sigc_exp : (T)0;
     const T smc = valid ? ct->smax[c] : (T)0;  // the cell's (sigma c)_max before this round
@@ -1809,6 +2016,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     // cell, so the outcome is that of the one-by-one loop.
     bool known = false;
     T ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cr = 0, sc = (T)-1;
+    NtcTest tt = {-1.0, 0.0f, false};
     while (pending) {
       const bool mine = (pending >> lane) & 1u;
       if (mine) {
@@ -1826,33 +2034,48 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         ax = svx[ci]; ay = svy[ci]; az = svz[ci];
         bx = svx[cj]; by = svy[cj]; bz = svz[cj];
         const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
-        cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
-        sc = coef * cpow(cr, ex);
+        if constexpr (sizeof(T) == 4) {
+          cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+          sc = coef * cpow(cr, ex);
+        } else {
+          const Geo<float>& G32 = inst_params<ONE>(a, ct->inst[c]).g32;
+          tt = ntc_test(g0, g1, g2, smc, coef, ex, G32.sigc_coef, G32.sigc_exp);
+          sc = tt.sc;
+        }
         known = true;
       }
       // inclusive prefix over the cell's lanes: maximum of the evaluated
       // sigma c, and whether all of them are evaluated
+      const bool all = !(~__ballot_sync(kFull, known) & upto & (0xFFFFFFFFu << seg0));
       T pm = known ? sc : (T)-1;
-      bool all = known;
+      // (FP64 mode: sigma c is formed only where it may exceed the maximum)
+      if (sizeof(T) == 4 || __any_sync(kFull, tt.exact)) {
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const T y = __shfl_up_sync(kFull, pm, o);
-        const int co = __shfl_up_sync(kFull, c, o);
-        const bool ya = __shfl_up_sync(kFull, all, o);
-        if (lane >= o && co == c) {
-          if (y > pm) pm = y;
-          all = all && ya;
+        for (int o = 1; o < 32; o <<= 1) {
+          const T y = __shfl_up_sync(kFull, pm, o);
+          if (lane - o >= seg0 && y > pm) pm = y;
         }
       }
       const T smL = pm > smc ? pm : smc;
       // P_c = sigma c / (sigma c)_max against u3; FP32 mode compares the
       // product (also monotone in (sigma c)_max, as the early rejection needs)
       bool pass;
-      if constexpr (sizeof(T) == 4) pass = ev && u3 * smL < sc;
-      else pass = ev && u3 < sc / smL;
+      if constexpr (sizeof(T) == 4) pass = ev && dr.u3 * smL < sc;
+      else pass = ev && ntc_pass(tt, dr, ax - bx, ay - by, az - bz, smc, smL, coef, ex);
       const bool decided = ev && (all || !pass);
       if (decided && pass) {
         atomicAdd(&ct->nacc[c], 1);
+        T u4, u5;
+        if constexpr (sizeof(T) == 4) {
+          u4 = dr.u4;
+          u5 = dr.u5;
+        } else {
+          const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
+          const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
+          cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+          u4 = dr.u4();
+          u5 = ntc_u5(step, (uint32_t)ct->kl[c], (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
+        }
         const T cchi = (T)2.0 * u4 - (T)1.0;
         const T schi = csqrt((T)1.0 - cchi * cchi);
         T sn, cs;
@@ -1871,11 +2094,12 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     }
     // the round's candidates raise the cell's (sigma c)_max
     T pm = sc;
+    if (sizeof(T) == 4 || __any_sync(kFull, tt.exact)) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T y = __shfl_up_sync(kFull, pm, o);
-      const int co = __shfl_up_sync(kFull, c, o);
-      if (lane >= o && co == c && y > pm) pm = y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(kFull, pm, o);
+        if (lane - o >= seg0 && y > pm) pm = y;
+      }
     }
     if (seg_last && pm > smc) ct->smax[c] = pm;
     __syncwarp();
@@ -1919,6 +2143,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       int s = lane < nlist ? stag[lane] : -1;
       int next = 32, t = 0, c = 0, armax = 1;
       T RT = 0, s2RT = 0, Amax = 0, omp = 0, q0 = 0, q1 = 0, q2 = 0, kA = 0, iRT = 0;
+      ShakhovFilter fl = {};
       Uni<T> r(0u, 0u, 0u, 0u, 0u, 0u);
       auto take = [&](int slot) {
         s = slot;
@@ -1939,13 +2164,15 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         q0 = ct->q[0][c];
         q1 = ct->q[1][c];
         q2 = ct->q[2][c];
+        if constexpr (sizeof(T) == 8) fl = shakhov_filter(RT, Amax, omp, q0, q1, q2);
       };
       take(s);
       while (__any_sync(kFull, s >= 0)) {
         bool done = false;
         if (s >= 0) {
           T C0, C1, C2;
-          const bool acc = shakhov_attempt<T>(r, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, &C0, &C1, &C2);
+          const bool acc = shakhov_attempt<T>(r, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, fl, t == armax - 1, &C0,
+                                              &C1, &C2);
           if (acc || t == armax - 1) {
             if (!acc) atomicAdd(&a.err[kErrAr], 1ull);
             atomicAdd(&ct->nar[c], t + 1);
@@ -2528,16 +2755,14 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
         const int g = base + tid;
         const bool valid = g < ncol;
         int ci = 0, cj = 0;
-        T u3 = 0, u4 = 0, u5 = 0;
+        NtcDraw<T> dr = {};
         if (valid) {
-          const NtcDraw<T> dr = ntc_draw((T)0, step, kl, (uint32_t)g, Pi.key0, Pi.key1);
-          u3 = dr.u3;
-          u4 = dr.u4;
-          u5 = dr.u5;
+          dr = ntc_draw((T)0, step, kl, (uint32_t)g, Pi.key0, Pi.key1);
           select_pair(N, dr.u1, dr.u2, tb->soff, nsub, &ci, &cj);
         }
         bool pending = valid, known = false;
         T ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cr = 0, sc = (T)-1;
+        NtcTest tt = {-1.0, 0.0f, false};
         for (;;) {
           if (pending) {
             atomicMin(&stag[ci], tid);
@@ -2554,8 +2779,13 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
             ax = svx[ci]; ay = svy[ci]; az = svz[ci];
             bx = svx[cj]; by = svy[cj]; bz = svz[cj];
             const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
-            cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
-            sc = coef * cpow(cr, ex);
+            if constexpr (sizeof(T) == 4) {
+              cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+              sc = coef * cpow(cr, ex);
+            } else {
+              tt = ntc_test(g0, g1, g2, smx, coef, ex, Pi.g32.sigc_coef, Pi.g32.sigc_exp);
+              sc = tt.sc;
+            }
             known = true;
           }
           // inclusive prefix over the candidates: maximum of the evaluated
@@ -2582,11 +2812,21 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
           }
           const T smL = pm > smx ? pm : smx;
           bool pass;
-          if constexpr (sizeof(T) == 4) pass = ev && u3 * smL < sc;
-          else pass = ev && u3 < sc / smL;
+          if constexpr (sizeof(T) == 4) pass = ev && dr.u3 * smL < sc;
+          else pass = ev && ntc_pass(tt, dr, ax - bx, ay - by, az - bz, smx, smL, coef, ex);
           const bool decided = ev && (all || !pass);
           if (decided && pass) {
             atomicAdd(&tb->nacc, 1);
+            T u4, u5;
+            if constexpr (sizeof(T) == 4) {
+              u4 = dr.u4;
+              u5 = dr.u5;
+            } else {
+              const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
+              cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
+              u4 = dr.u4();
+              u5 = ntc_u5(step, kl, (uint32_t)g, Pi.key0, Pi.key1);
+            }
             const T cchi = (T)2.0 * u4 - (T)1.0;
             const T schi = csqrt((T)1.0 - cchi * cchi);
             T sn, cs;
@@ -2628,6 +2868,7 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
         kA = omp / ((T)5.0 * RT * RT);
         iRT = (T)1.0 / RT;
       }
+      const ShakhovFilter fl = shakhov_filter(RT, Amax, omp, q0, q1, q2);
       int nres = 0, nar = 0;
       for (int s = tid; s < N; s += kHugeThreads) {
         const Uni<T> r0(step, kl, (uint32_t)s, kPurpShk << 24, Pi.key0, Pi.key1);
@@ -2637,7 +2878,8 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
         if (a.resamp) a.resamp[p0 + s] = 1;
         for (int t = 0;; ++t) {
           T C0, C1, C2;
-          const bool acc = shakhov_attempt<T>(r0, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, &C0, &C1, &C2);
+          const bool acc = shakhov_attempt<T>(r0, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, fl, t == Pi.ar_max - 1,
+                                              &C0, &C1, &C2);
           if (acc || t == Pi.ar_max - 1) {
             if (!acc) atomicAdd(&a.err[kErrAr], 1ull);
             nar += t + 1;
@@ -2880,14 +3122,24 @@ __global__ void __launch_bounds__(kFlightThreads, sizeof(T) == 4 ? 4 : 3) k_flig
           hit = true;
           if (!gone) key = (uint32_t)(P.cell_off + kl);
         } else {
-          bool gone = false;
-          if (!flight_fast<T, DIM>(P, x, v, dt)) {
-            const uint32_t c = ONE ? a.key_in[og[0]] : cg[0];
-            gone = move_particle<T, DIM>(P, a.surf, x, v, dt, step, kPurpWall, (uint32_t)(c - P.cell_off),
-                                         (uint32_t)(s - a.start[c]), 0u, a.err);
-            hit = true;
+          bool gone = false, clear = false;
+          if constexpr (sizeof(T) == 8) {
+            clear = flight_clear<DIM>(P, x, v, dt);
+            if (clear) {
+#pragma unroll
+              for (int d = 0; d < DIM; ++d) x[d] += v[d] * dt;
+              key = (uint32_t)P.cell_off + cell_of_clear<DIM>(P, x);
+            }
           }
-          if (!gone) key = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
+          if (!clear) {
+            if (!flight_fast<T, DIM>(P, x, v, dt)) {
+              const uint32_t c = ONE ? a.key_in[og[0]] : cg[0];
+              gone = move_particle<T, DIM>(P, a.surf, x, v, dt, step, kPurpWall, (uint32_t)(c - P.cell_off),
+                                           (uint32_t)(s - a.start[c]), 0u, a.err);
+              hit = true;
+            }
+            if (!gone) key = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
+          }
         }
 #pragma unroll
         for (int d = 0; d < DIM; ++d) ((T*)a.Bpos[d])[s] = x[d];
