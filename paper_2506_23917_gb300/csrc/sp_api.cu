@@ -174,6 +174,10 @@ void fill_params(const sp_config& c, InstParams* P, int64_t cell_off) {
   P->tau_k = c.mu_ref * pow(c.T_ref, -c.omega) / (c.m * c.R);
   P->inv_tau_k = 1.0 / P->tau_k;
   P->omf = (float)(1.0 - c.omega);
+  P->inv3R_f = (float)P->inv3R;
+  P->gR_f = (float)(c.gamma * c.R);
+  P->Fn_itau_f = (float)(c.Fn * P->inv_tau_k);
+  P->hFn_f = (float)(0.5 * c.Fn);
   P->inv_Lmin = 1.0 / P->Lmin;
   P->inv_Fn = 1.0 / c.Fn;
   for (int d = 0; d < 3; ++d) {

@@ -66,6 +66,15 @@ __device__ __forceinline__ float u01f(uint32_t a) {
   return (float)(2u * (a >> 9) + 1u) * 5.9604644775390625e-8f;
 }
 
+// An FP32 value widened exactly, by integer operations (the conversion
+// instruction goes through the FP64 pipe); subnormals take the instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+  if ((m < 0x00800000u && m != 0u) || m >= 0x7F800000u) return (double)x;
+  const uint32_t hi = m ? (u & 0x80000000u) | ((m >> 3) + 0x38000000u) : u;
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
 // A uniform stream addressed by (step, a, b, purpose<<24 | sub); the q-th
 // uniform lives in block q/2 (FP64) or q/4 (FP32) of the counter word 3.
 template <class T>
@@ -106,31 +115,6 @@ struct Uni<float> {
   }
 };
 
-// N consecutive uniforms q0 .. q0+N-1 of a stream (the same values as
-// Uni<T>::get), for draws whose index is only known at run time: the
-// blocks they span are produced by a loop around one inlined Philox body
-// instead of one inlined body per draw.
-__device__ __forceinline__ float uni_word(const uint4& w, int r, float) {
-  return u01f(r == 0 ? w.x : r == 1 ? w.y : r == 2 ? w.z : w.w);
-}
-__device__ __forceinline__ double uni_word(const uint4& w, int r, double) {
-  return r ? u01d(w.z, w.w) : u01d(w.x, w.y);
-}
-template <class T, int N>
-__device__ __forceinline__ void uni_run(const Uni<T>& u, int q0, T (&out)[N]) {
-  constexpr int per = sizeof(T) == 8 ? 2 : 4;
-  const int b0 = q0 / per, b1 = (q0 + N - 1) / per;
-#pragma unroll 1
-  for (int b = b0; b <= b1; ++b) {
-    const uint4 w = philox10(u.c0, u.c1, u.c2, u.c3 + (uint32_t)b, u.k0, u.k1);
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      const int q = q0 + j;
-      if (q / per == b) out[j] = uni_word(w, q % per, (T)0);
-    }
-  }
-}
-
 // Asynchronous global -> shared copy of one 4- or 8-byte element (no
 // register staging), and the wait for all of this thread's copies.
 template <int BYTES>
@@ -139,8 +123,6 @@ __device__ __forceinline__ void cp_async(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(gsrc), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-// Request a global line into L2 (no register result, nothing waits on it).
-__device__ __forceinline__ void prefetch_l2(const void* g) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(g)); }
 
 // ---------------------------------------------------------------------------
 // Precision helpers
@@ -861,7 +843,7 @@ struct __align__(16) CellTab {
   uint16_t soff[32][kMaxSub + 1];  // sub-cell offsets within each cell (sub-cells on)
   T U[3][32];
   T q[3][32];
-  T RT[32], s2RT[32], Amax[32], Pres[32], omp[32], dt[32];
+  T RT[32], s2RT[32], Amax[32], Pres[32], omp[32];
   // Conservation rescale c' = U + (c - U_p) f, applied slot by slot.
   // T == A: Up = U_p and f.  Mixed precision: the same map written as
   // c' = c f + K with f = f[] + fl[] and K = Up[] + Kl[] as FP32 pairs
@@ -977,7 +959,7 @@ struct ExactSum {
     r.e = __shfl_sync(kFull, e, src);
     return r;
   }
-  __device__ __forceinline__ double get() const { return (double)s + (double)e; }
+  __device__ __forceinline__ double get() const { return widen(s) + widen(e); }
 };
 template <class T, class A>
 using CellAcc = typename std::conditional<mixed_prec<T, A>(), ExactSum, PlainSum<T>>::type;
@@ -1042,10 +1024,12 @@ struct LanePart {
   static constexpr int split = kSplit;
   int c, b, e;
   int own_parts, h0;
+  uint16_t* scratch;  // [32] shared, for the FP64 sums
 };
 template <>
 struct LanePart<0> {
   static constexpr int split = 0;
+  uint16_t* scratch;
 };
 
 // The lanes' parts of a batch of G cells (cells with Ni > kLaneSumMax: one
@@ -1054,6 +1038,7 @@ struct LanePart<0> {
 template <int split, class TabT>
 __device__ __forceinline__ LanePart<split> lane_parts(TabT* ct, int G, bool own, int offi, int Ni) {
   LanePart<split> lp;
+  lp.scratch = ct->hpart;
   if constexpr (split == 0) {
     return lp;
   } else {
@@ -1100,6 +1085,13 @@ __device__ __forceinline__ LanePart<split> lane_parts(TabT* ct, int G, bool own,
   }
 }
 
+// Lanes that share the FP64 sum of a cell of n particles (a power of two,
+// about eight particles each).
+__device__ __forceinline__ int fp64_lanes(int n) {
+  const int q = (n + 7) >> 3;  // ceil(n / 8), rounded up to a power of two
+  return q <= 1 ? 1 : 1 << (32 - __clz(q - 1));
+}
+
 // kLo: the terms come with exact low parts (else lo is ignored).
 template <class Acc, int K, bool kLo = false, class LP, class F>
 __device__ __forceinline__ void cell_sums_acc(const LP& lp, bool own, int offi, int Ni, Acc (&out)[K], F f) {
@@ -1108,9 +1100,62 @@ __device__ __forceinline__ void cell_sums_acc(const LP& lp, bool own, int offi, 
   const bool small = own && Ni <= lane_sum_max<Acc>;
 #pragma unroll
   for (int k = 0; k < K; ++k) out[k].init();
-  if constexpr (sizeof(Tm) == 8 || LP::split == 0) {
-    // FP64 terms (FP64 mode; the FP32 mode's FP64 record sums), or no
-    // split parts: one lane per cell, in slot order
+  if constexpr (sizeof(Tm) == 8) {
+    // FP64 terms (FP64 mode; the FP32 mode's FP64 record sums): an FP64
+    // instruction holds the pipe as long for one lane as for 32, so a cell's
+    // slots are dealt to P = fp64_lanes(N) neighbouring lanes (every P-th
+    // slot each, then a tree over the P lanes), as many cells at a time as
+    // fill the warp
+    const int P = small && Ni > 0 ? fp64_lanes(Ni) : 0;
+    int incl = P;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    for (unsigned todo = __ballot_sync(kFull, P > 0); todo;) {
+      const int first = __ffs(todo) - 1;
+      const int before = __shfl_sync(kFull, incl - P, first);
+      const bool fit = P > 0 && lane >= first && incl - before <= 32;
+      const unsigned round = __ballot_sync(kFull, fit);
+      const int start = incl - P - before;  // the cell's first lane
+      const unsigned heads = __reduce_or_sync(kFull, fit ? 1u << start : 0u);
+      const int tot = __shfl_sync(kFull, incl, 31 - __clz((int)round)) - before;
+      if (fit) lp.scratch[start] = (uint16_t)lane;
+      __syncwarp();
+      const int hs = 31 - __clz((int)(heads & (0xFFFFFFFFu >> (31 - lane)))), p = lane - hs;
+      const int c = lp.scratch[hs];
+      const int o0 = __shfl_sync(kFull, offi, c), n = __shfl_sync(kFull, Ni, c), Pc = __shfl_sync(kFull, P, c);
+      Acc acc[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) acc[k].init();
+      if (lane < tot)
+        for (int s = o0 + p; s < o0 + n; s += Pc) {
+          Tm v[K], lo[K];
+          f(s, c, v, lo);
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            if constexpr (kLo) acc[k].add(v[k], lo[k]);
+            else acc[k].add1(v[k]);
+          }
+        }
+      const int pmax = (int)__reduce_max_sync(kFull, (unsigned)P & (fit ? ~0u : 0u));
+      for (int o = pmax >> 1; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const Acc y = acc[k].shfl_from(lane + o < 32 ? lane + o : lane);
+          if (o < Pc && p < o) acc[k].combine(y);
+        }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const Acc y = acc[k].shfl_from(fit ? start : lane);
+        if (fit) out[k] = y;
+      }
+      todo &= ~round;
+      __syncwarp();
+    }
+  } else if constexpr (LP::split == 0) {
+    // no split parts: one lane per cell, in slot order
     if (small) {
       for (int s = offi; s < offi + Ni; ++s) {
         Tm v[K], lo[K];
@@ -1530,10 +1575,40 @@ __device__ __forceinline__ bool shakhov_surely_rejected(const uint32_t* wa, cons
   return lim * 0.99999f > A + err + 1e-5f;
 }
 
+// The words of attempt t's five uniforms: uniform q = 1 + 5 t + j in half
+// q & 1 of block q / 2.
+template <class U>
+__device__ __forceinline__ void shakhov_words(const U& r, int t, uint32_t* wa, uint32_t* wb) {
+  const int q0 = 1 + 5 * t;
+#pragma unroll 1
+  for (int b = q0 >> 1; b <= (q0 + 4) >> 1; ++b) {
+    const uint4 w = philox10(r.c0, r.c1, r.c2, r.c3 + (uint32_t)b, r.k0, r.k1);
+#pragma unroll
+    for (int j = 0; j < 5; ++j)
+      if ((q0 + j) >> 1 == b) {
+        wa[j] = (q0 + j) & 1 ? w.z : w.x;
+        wb[j] = (q0 + j) & 1 ? w.w : w.y;
+      }
+  }
+}
+// The first attempt from t on that the filter does not reject (FP64 mode; the
+// last one, armax - 1, is kept whatever it is): the lanes of a warp then take
+// their FP64 attempts together.
+template <class T>
+__device__ __forceinline__ int shakhov_skip(const Uni<T>& r, int t, int armax, const ShakhovFilter& fl) {
+  if constexpr (sizeof(T) == 8) {
+    for (; t < armax - 1; ++t) {
+      uint32_t wa[5], wb[5];
+      shakhov_words(r, t, wa, wb);
+      if (!shakhov_surely_rejected(wa, wb, fl)) break;
+    }
+  }
+  return t;
+}
+
 template <class T>
 __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, T Amax, T omp, T RT, T kA, T iRT,
-                                                T q0, T q1, T q2, const ShakhovFilter& fl, bool last, T* C0, T* C1,
-                                                T* C2) {
+                                                T q0, T q1, T q2, T* C0, T* C1, T* C2) {
   T R1, R2, R3, R4, R5;
   if constexpr (sizeof(T) == 4) {
     const uint4 w = philox10(r.c0, r.c1, r.c2, r.c3 + 1u + (uint32_t)t, r.k0, r.k1);
@@ -1543,20 +1618,8 @@ __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, 
     R3 = (float)(2u * (w.z & 0xFFFFu) + 1u) * 7.62939453125e-6f;
     R5 = u01f(w.w);
   } else {
-    // the words of the five uniforms: uniform q in half q & 1 of block q / 2
     uint32_t wa[5], wb[5];
-    const int q0u = 1 + 5 * t;
-#pragma unroll 1
-    for (int b = q0u >> 1; b <= (q0u + 4) >> 1; ++b) {
-      const uint4 w = philox10(r.c0, r.c1, r.c2, r.c3 + (uint32_t)b, r.k0, r.k1);
-#pragma unroll
-      for (int j = 0; j < 5; ++j)
-        if ((q0u + j) >> 1 == b) {
-          wa[j] = (q0u + j) & 1 ? w.z : w.x;
-          wb[j] = (q0u + j) & 1 ? w.w : w.y;
-        }
-    }
-    if (!last && shakhov_surely_rejected(wa, wb, fl)) return false;  // (the last one is kept whatever it is)
+    shakhov_words(r, t, wa, wb);
     R1 = u01d(wa[0], wb[0]); R2 = u01d(wa[1], wb[1]); R3 = u01d(wa[2], wb[2]);
     R4 = u01d(wa[3], wb[3]); R5 = u01d(wa[4], wb[4]);
   }
@@ -1573,6 +1636,40 @@ __device__ __forceinline__ bool shakhov_attempt(const Uni<T>& r, int t, T s2RT, 
   if constexpr (sizeof(T) == 4) A = (T)1.0 + kA * qC * (CC * iRT - (T)5.0);
   else A = (T)1.0 + omp * qC / ((T)5.0 * RT * RT) * (CC / RT - (T)5.0);
   return R5 * Amax < A;
+}
+
+// Mixed precision: the outcome of cell_math_lean for a cell whose decisions
+// FP32 estimates settle -- a pure DSMC split (Delta t_c well below tau), a
+// Delta t_c well above the smallest found so far, and a candidate count whose
+// fractional draw is not close to an integer.  The estimates' relative
+// errors (sums of a dozen roundings, __powf's 1e-5) stay below 3e-5.  A
+// batch whose cells are all settled skips the FP64 arithmetic (60 to 130
+// operations of the FP64 pipe in one dependent chain).  s: the cell's sums of
+// c; S2: of |C|^2 (high parts of the exact pairs).
+__device__ __forceinline__ bool cell_settled(const InstParams& Pi, uint32_t kl, int Ni, const float* s, float S2,
+                                             double iV, const double* iLc, int64_t kc, float smaxT, double dt_cur,
+                                             unsigned long long dt_min, uint32_t step, CellMath<double>& o) {
+  if (Pi.mode == 2 || Pi.ntc_carry || Ni < 2) return false;
+  const float fN = (float)Ni, iN = 1.0f / fN;
+  const float ux = s[0] * iN, uy = s[1] * iN, uz = s[2] * iN;
+  const float T = S2 * Pi.inv3R_f / (fN - 1.0f);
+  const float iL = approx_f32(iLc ? iLc[kc] : Pi.inv_Lmin);
+  const float idtc = (sqrtf(ux * ux + uy * uy + uz * uz) + sqrtf(Pi.gR_f * T)) * iL;  // 1 / Delta t_c
+  // (1 / Delta t_c above 0.999 of the largest so far: the FP64 value counts)
+  const float lim = 1.0f / approx_f32(__longlong_as_double((long long)dt_min));
+  const float nv = fN * approx_f32(iV);
+  bool ok = T > 1e-30f && T < 1e30f && idtc > 1e-30f && idtc < 1e30f && idtc < 0.999f * lim;
+  if (Pi.mode == 0) {
+    const float k = nv * Pi.Fn_itau_f * __powf(T, Pi.omf);  // 1 / tau
+    ok = ok && k > 1e-30f && k < 0.98f * idtc;
+  }
+  if (!ok) return false;
+  const float ncr = Pi.hFn_f * (fN - 1.0f) * nv * smaxT * approx_f32(dt_cur);
+  Uni<float> rr(step, kl, kSentinel, kPurpNtc << 24, Pi.key0, Pi.key1);
+  const float x = ncr + rr.get(0), f = floorf(x), m = 1e-4f * x + 1e-6f;
+  if (!(ncr > 1e-30f && x < 4096.0f && x - f > m && x - f < 1.0f - m)) return false;
+  o.ncol = (int64_t)(int)f;
+  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -1598,7 +1695,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   int Ni = 0, offi = 0;
   uint32_t inst = 0;
   // loaded early: used by the cell math (mixed precision: 1/V)
-  double vol_k = 1.0, smax_k = 0.0;
+  double vol_k = 1.0, smax_k = 0.0, dt_k = 0.0;
+  unsigned long long dt_min_k = 0;  // the instance's minimum so far
   if (own) {
     vol_k = kMixed ? a.ivol[kc] : a.vol[kc];
     smax_k = a.smax[kc];
@@ -1606,6 +1704,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     Ni = (int)(a.start[kc + 1] - s0);
     offi = (int)(s0 - p0);
     inst = a.cell_inst[kc];
+    dt_k = a.dt_cur[inst];
+    if constexpr (kMixed) dt_min_k = *(volatile const unsigned long long*)&a.dt_min[inst];
     ct->off[lane] = offi;
     ct->inst[lane] = (int)inst;
     ct->kl[lane] = (int)(kc - inst_params<ONE>(a, inst).cell_off);
@@ -1701,6 +1801,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   // both passes summed without loss into FP64).
   bool one_pass = false;
   A m0 = 0, m1 = 0, m2 = 0, mS2 = 0, mS3x = 0, mS3y = 0, mS3z = 0;
+  float sum_h[4] = {0, 0, 0, 0};  // mixed precision: the sums' high parts
   if constexpr (sizeof(A) == 4) {
     one_pass = own && Ni > 0 && Ni <= kLaneSumMax;
     if (one_pass) {
@@ -1776,8 +1877,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     // the second pass: sum |C|^2 and sum |C|^2 C (mixed precision: sum |C|^2
     // only; sum |C|^2 C, needed by the Shakhov cells alone, after Step 4)
     constexpr int K2 = kMixed ? 1 : 4;
-    A r2[K2];
-    cell_sums<Acc, K2>(lp, two_pass, offi, Ni, r2, [&](int s, int c, T* v, T* lo) {
+    Acc a2[K2];
+    cell_sums_acc<Acc, K2>(lp, two_pass, offi, Ni, a2, [&](int s, int c, T* v, T* lo) {
       T C0 = svx[s] - ct->Up[0][c], C1 = svy[s] - ct->Up[1][c], C2 = svz[s] - ct->Up[2][c];
       if constexpr (kMixed) {
         C0 -= ct->Kl[0][c];
@@ -1799,12 +1900,17 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       m1 = r1[1];
       m2 = r1[2];
       if (Ni >= 2) {
-        mS2 = r2[0];
+        mS2 = a2[0].get();
         if constexpr (K2 == 4) {
-          mS3x = r2[1];
-          mS3y = r2[2];
-          mS3z = r2[3];
+          mS3x = a2[1].get();
+          mS3y = a2[2].get();
+          mS3z = a2[3].get();
         }
+      }
+      if constexpr (kMixed) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sum_h[d] = a1[d].s;
+        sum_h[3] = a2[0].s;
       }
     }
     __syncwarp();
@@ -1818,9 +1924,13 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   if (own) {
     sample = (int64_t)step >= (int64_t)Pi.n_steady;
     smaxT = (T)smax_k;
-    cell_math<T, A, !kMixed>(a, Pi, kc, (uint32_t)ct->kl[lane], Ni, m0, m1, m2, mS2, mS3x, mS3y, mS3z, vol_k,
-                             smaxT, a.dt_cur[inst], step, cm);
-    ct->dt[lane] = (T)cm.dtG;
+    bool settled = false;
+    if constexpr (kMixed)
+      settled = cell_settled(Pi, (uint32_t)ct->kl[lane], Ni, sum_h, sum_h[3], vol_k, a.iLc, kc, smaxT, dt_k, dt_min_k,
+                             step, cm);
+    if (!settled)
+      cell_math<T, A, !kMixed>(a, Pi, kc, (uint32_t)ct->kl[lane], Ni, m0, m1, m2, mS2, mS3x, mS3y, mS3z, vol_k,
+                               smaxT, dt_k, step, cm);
     ct->Pres[lane] = 0;
     if (cm.shk) {
       ct->RT[lane] = (T)cm.RT;
@@ -2171,8 +2281,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         bool done = false;
         if (s >= 0) {
           T C0, C1, C2;
-          const bool acc = shakhov_attempt<T>(r, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, fl, t == armax - 1, &C0,
-                                              &C1, &C2);
+          t = shakhov_skip(r, t, armax, fl);
+          const bool acc = shakhov_attempt<T>(r, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, &C0, &C1, &C2);
           if (acc || t == armax - 1) {
             if (!acc) atomicAdd(&a.err[kErrAr], 1ull);
             atomicAdd(&ct->nar[c], t + 1);
@@ -2200,8 +2310,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   const int nres_i = own ? ct->nres[lane] : 0;
   const unsigned rcells = __ballot_sync(kFull, nres_i > 0);
   const bool rown = own && nres_i > 0;
-  // Step 5 squares of the post-collision velocities of a rescaled cell
-  // (mixed precision: exact from the rescale's sums; else phase 8's pass)
+  // Step 5 squares of the post-collision velocities of a rescaled cell (FP64
+  // cells: from the rescale; else phase 8's pass)
   A bsq[3] = {0, 0, 0};
   if (rcells) {
     if constexpr (!kMixed) {
@@ -2228,6 +2338,14 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       if (rown) {
         const double Tp = (double)r2[0] / (3.0 * Pi.R * (double)(Ni - 1));
         ct->f[lane] = Tp > 0 ? (T)sqrt((double)TA / Tp) : (T)-1;
+        if constexpr (sizeof(A) == 8) {  // (T_p = 0: not rescaled, every velocity is U_p)
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const A u = Tp > 0 ? UA[d] : (A)ct->Up[d][lane];
+            bsq[d] = (A)Ni * u * u;
+          }
+          if (Tp > 0) bsq[0] += (A)3.0 * (A)Pi.R * (A)(Ni - 1) * TA;
+        }
       }
       __syncwarp();
       for (int s = lane; s < M; s += 32) {
@@ -2346,16 +2464,19 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   }
   // ---- 8. time-averaged sums (Step 5).  Both collision sub-steps conserve
   // each cell's momentum (the DSMC pair rule and the rescale to U), so the
-  // momentum sums are those of Step 3 up to rounding; the per-component
-  // squares need a pass over the post-collision velocities.  Mixed mode:
-  // only sum |c|^2 is kept, in the first square's slot (the averaged T
-  // needs no more): a rescaled cell's comes exact from the rescale's sums,
-  // and a cell without a rescale had DSMC collisions alone, which conserve
-  // its energy, so its sum is sum |C|^2 + |sum c|^2 / N of Step 3.
-  const bool need_sq = !kMixed && own && sample && Ni > 0;
+  // momentum sums are those of Step 3 up to rounding.  With FP64 cells (FP64
+  // and mixed mode) only the total sum |c|^2 is kept, in the first square's
+  // slot (the averaged T needs no more): a cell without a rescale had DSMC
+  // collisions alone, which conserve its energy, so its total is
+  // sum |C|^2 + |sum c|^2 / N of Step 3; a rescaled cell's comes from the
+  // rescale (mixed: its exact sums; FP64: its targets, sum |c'|^2 =
+  // 3 R (N-1) T + N |U|^2).  The all-FP32 mode sums the per-component squares
+  // of the post-collision velocities.
+  constexpr bool kEnergy = sizeof(A) == 8;
+  const bool need_sq = !kEnergy && own && sample && Ni > 0;
   const A a0 = m0, a1 = m1, a2 = m2;
   A b0 = bsq[0], b1 = bsq[1], b2 = bsq[2];
-  if constexpr (kMixed) {
+  if constexpr (kEnergy) {
     if (own && sample && Ni > 0) {
       if (nres_i > 0) {
         b0 = b0 + b1 + b2;
@@ -2366,7 +2487,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       b1 = b2 = 0;
     }
   }
-  constexpr unsigned kSampSlots = kMixed ? 0x9Fu : 0xFFu;  // mixed: slots 5, 6 unused
+  constexpr unsigned kSampSlots = kEnergy ? 0x9Fu : 0xFFu;  // FP64 cells: slots 5, 6 unused
   double sv[8];  // the accumulators, requested before the sums
   if (own && sample) {
 #pragma unroll
@@ -2374,8 +2495,6 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   }
   if (__any_sync(kFull, need_sq)) {
     A r[3];
-    // (mixed precision: the FP32 squares, each rounded as the FP32 state
-    // itself is, summed without loss; exact squares cost 1.6 %)
     cell_sums<Acc, 3>(lp, need_sq, offi, Ni, r, [&](int s, int c, T* v, T* lo) {
       const T x0 = svx[s], x1 = svy[s], x2 = svz[s];
       v[0] = x0 * x0;
@@ -2398,7 +2517,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         S[2 * NC + kc] = sv[2] + (double)a1;
         S[3 * NC + kc] = sv[3] + (double)a2;
         S[4 * NC + kc] = sv[4] + (double)b0;
-        if constexpr (!kMixed) {
+        if constexpr (!kEnergy) {
           S[5 * NC + kc] = sv[5] + (double)b1;
           S[6 * NC + kc] = sv[6] + (double)b2;
         }
@@ -2427,7 +2546,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
 }
 
 template <class T, class A, int DIM, bool ONE>
-__global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, 1) k_collide(StepArgs a, int big) {
+__global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1) k_collide(StepArgs a, int big) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cap = big ? a.big_cap : a.cap_small;
@@ -2878,8 +2997,8 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
         if (a.resamp) a.resamp[p0 + s] = 1;
         for (int t = 0;; ++t) {
           T C0, C1, C2;
-          const bool acc = shakhov_attempt<T>(r0, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, fl, t == Pi.ar_max - 1,
-                                              &C0, &C1, &C2);
+          t = shakhov_skip(r0, t, Pi.ar_max, fl);
+          const bool acc = shakhov_attempt<T>(r0, t, s2RT, Amax, omp, RT, kA, iRT, q0, q1, q2, &C0, &C1, &C2);
           if (acc || t == Pi.ar_max - 1) {
             if (!acc) atomicAdd(&a.err[kErrAr], 1ull);
             nar += t + 1;

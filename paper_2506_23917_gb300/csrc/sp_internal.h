@@ -13,8 +13,8 @@ constexpr int kMaxCross = 4096;              // face crossings per particle per 
 // particles is summed by lanes of its batch's warp, above it by the whole
 // warp.  With an FP32 state in 2-D such a cell takes ceil(N / kSplitLanes) lanes
 // (at most kMaxParts), each summing a contiguous part; the batch plan keeps
-// the lanes of a batch within 32.  FP64 mode: one lane per cell (the
-// oracle's summation order).  (Developed cylinder, 864 x 2: split 32 +2.5 %
+// the lanes of a batch within 32.  FP64 mode: about eight particles per
+// lane, as many cells at a time as fill the warp (cell_sums_acc).  (Developed cylinder, 864 x 2: split 32 +2.5 %
 // over no split; 16 / 24 / 48 / 64 and 8 parts were slower than 32 -- more
 // lanes per cell leave fewer cells per batch.)
 constexpr int kLaneSumMax = 256;
@@ -87,6 +87,7 @@ struct InstParams {
   double inv_Lmin;   // 1 / L_min
   double inv_Fn;     // 1 / F_N
   float omf;         // 1 - omega in FP32 (the bound that certifies a pure DSMC split)
+  float inv3R_f, gR_f, Fn_itau_f, hFn_f;  // inv3R, gamma R, F_N / tau_k, F_N / 2 in FP32 (estimates)
   // body-fitted O-grid (mesh = 1): n[0] radial layers x n[1] sectors, mnl
   // reservoir rings; its nodes start at mnode_off (node (i, j) at
   // mnode_off + i n[1] + j) and its radii at mrad_off
