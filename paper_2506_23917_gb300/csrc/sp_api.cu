@@ -100,6 +100,7 @@ struct sp_ctx {
   uint32_t hM = 0;
   // body-fitted O-grid instances (all instances share the mesh kind)
   int mesh = 0;
+  bool subcells = false;  // an instance uses sub-cells
   double *Lc = nullptr, *iLc = nullptr, *mrad = nullptr;  // [NC], [NC], radii
   void *mface = nullptr, *mnode = nullptr;                 // state type
 };
@@ -468,6 +469,7 @@ StepArgs make_step_args(sp_ctx* c, int par) {
   a.cap_small = c->sched_cap;
   a.surf = c->n_surf_tot > 0 ? c->surf : nullptr;
   a.one = c->n_inst == 1 ? 1 : 0;
+  a.subcells = c->subcells ? 1 : 0;
   a.P0 = c->hP[0];
   return a;
 }
@@ -515,10 +517,9 @@ bool apply_schedule(sp_ctx* c, int cap, int warps) {
   if (cap < 32 || cap > kHugeCell || warps < 1 ||
       warps > kMaxWarpsPerBlock)
     return false;
-  const size_t smem = c->K->collide_smem(warps, cap);
-  if (smem > (size_t)kMaxDynSmem) return false;
+  if (!c->K->collide_fits(warps, cap)) return false;
   const bool one = c->n_inst == 1;
-  const int per_sm = c->K->collide_blocks_per_sm(c->dim, warps, cap, one);
+  const int per_sm = c->K->collide_blocks_per_sm(c->dim, warps, cap, one, c->subcells);
   if (per_sm < 1) return false;
   c->sched_cap = cap;
   c->sched_warps = warps;
@@ -791,6 +792,7 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
     off += c->hP[i].ncells;
     c->hP[i].surf_off = soff;
     soff += c->hP[i].n_surf;
+    if (c->hP[i].nsub > 1) c->subcells = true;
   }
   c->n_surf_tot = soff;
   c->NC = off;
@@ -1118,7 +1120,7 @@ sp_status sp_autotune(sp_ctx* c, int steps_per_trial, int* cap_out, int* warps_o
     for (int ci : caps) sched.push_back({ci, wi});
     int last = -1;
     for (int ci = kHugeCell; ci >= 128; ci -= 32) {
-      const int per = c->K->collide_blocks_per_sm(c->dim, wi, ci, c->n_inst == 1);
+      const int per = c->K->collide_blocks_per_sm(c->dim, wi, ci, c->n_inst == 1, c->subcells);
       if (per != last && per > 0 &&
           std::find(sched.begin(), sched.end(), std::make_pair(ci, wi)) == sched.end())
         sched.push_back({ci, wi});

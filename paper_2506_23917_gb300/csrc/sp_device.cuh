@@ -833,16 +833,15 @@ template <class T, class A>
 struct __align__(16) CellTab {
   int off[33];   // slot range of cell i: [off[i], off[i+1])
   int inst[32];
-  int kl[32];    // instance-local cell index (Philox counter)
+  uint8_t ne[32];  // the cells that hold particles, in order
   int nres[32];
   int nar[32];
   int nacc[32];
   int coff[33];  // candidate offsets of the flattened NTC loop
   int pad[2];
   uint16_t hpart[32];  // helper lane -> (cell << 8 | part) of the split sums
-  uint16_t soff[32][kMaxSub + 1];  // sub-cell offsets within each cell (sub-cells on)
   T U[3][32];
-  T q[3][32];
+  T q[3][32];    // (from the rescale on: its factor f, high and low part, in q[0], q[1])
   T RT[32], s2RT[32], Amax[32], Pres[32], omp[32];
   // Conservation rescale c' = U + (c - U_p) f, applied slot by slot.
   // T == A: Up = U_p and f.  Mixed precision: the same map written as
@@ -851,26 +850,29 @@ struct __align__(16) CellTab {
   // of the second moment pass uses Up / Kl the same way (U = Up + Kl).
   T Up[3][32];
   T Kl[3][32];
-  T f[32];
-  T fl[32];
   T smax[32];    // (sigma_T c_r)_max while candidates run
 };
 
-// Staging per particle: velocities (3 T), source index, clash tag, cell.
-// In FP32 modes the source indices live in the x-velocity array until the
-// gather overwrites them slot by slot (the free flight re-reads them from
-// perm), which saves 4 bytes per particle and raises the resident warps.
+// Staging per particle: velocities (3 T), source index, and two bytes that
+// hold the NTC clash tags (a table of cap / 2 words that the slots are folded
+// into), then the list of resampled slots.  In FP32 modes the source indices
+// live in the x-velocity array until the gather overwrites them slot by slot.
+// 14 bytes per particle (FP32) let 16 warps of 812 particles share an SM;
+// with 4-byte tags and a cell byte per slot (17) it was 12 of 864.
 template <class T>
 __host__ __device__ constexpr bool idx_in_velocity() {
   return sizeof(T) == 4;
 }
 template <class T>
 __host__ __device__ constexpr size_t stage_bytes_per_particle() {
-  return 3 * sizeof(T) + (idx_in_velocity<T>() ? 0 : 4) + 4 + 1;
+  return 3 * sizeof(T) + (idx_in_velocity<T>() ? 0 : 4) + 2;
 }
+// sub-cells on: their offsets within each cell of the batch
+constexpr size_t kSubBytes = 32 * (kMaxSub + 1) * sizeof(uint16_t);
 template <class T, class A>
-__host__ __device__ constexpr size_t warp_stage_bytes(int cap) {
-  return (sizeof(CellTab<T, A>) + (size_t)cap * stage_bytes_per_particle<T>() + 15) / 16 * 16;
+__host__ __device__ constexpr size_t warp_stage_bytes(int cap, bool subcells) {
+  return (sizeof(CellTab<T, A>) + (subcells ? kSubBytes : 0) + ((size_t)cap * stage_bytes_per_particle<T>() + 3) / 4 * 4 +
+          15) / 16 * 16;
 }
 
 // ---------------------------------------------------------------------------
@@ -1681,7 +1683,7 @@ __device__ __forceinline__ bool cell_settled(const InstParams& Pi, uint32_t kl, 
 // ---------------------------------------------------------------------------
 template <class T, class A, int DIM, bool ONE>
 __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A>* ct, uint32_t* sidx,
-                              int* stag, uint8_t* sseg, T* svx, T* svy, T* svz) {
+                              int* tags, int ntag, uint16_t (*soff)[kMaxSub + 1], T* svx, T* svy, T* svz) {
   using Acc = CellAcc<T, A>;
   constexpr bool kMixed = mixed_prec<T, A>();
   const int lane = threadIdx.x & 31;
@@ -1708,7 +1710,6 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     if constexpr (kMixed) dt_min_k = *(volatile const unsigned long long*)&a.dt_min[inst];
     ct->off[lane] = offi;
     ct->inst[lane] = (int)inst;
-    ct->kl[lane] = (int)(kc - inst_params<ONE>(a, inst).cell_off);
     ct->nres[lane] = 0;
     ct->nar[lane] = 0;
   }
@@ -1718,19 +1719,24 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   const auto lp = lane_parts<kSplitOf<T, DIM>>(ct, G, own, offi, Ni);
   // ---- 1. source indices (in source order within each cell when the run is
   // reproducible: k_order) and cell of each slot
-  // (the index copies run while the cell of each slot is written)
 #pragma unroll 4
   for (int s = lane; s < M; s += 32) cp_async<4>(&sidx[s], &a.perm[p0 + s]);
-  // each lane writes its own cell's slots (one pass for all cells of the
-  // batch instead of one warp-wide pass per cell); cells above
-  // kLaneSumMax particles are written by the whole warp
-  if (own && Ni <= kLaneSumMax)
-    for (int s = offi; s < offi + Ni; ++s) sseg[s] = (uint8_t)lane;
-  for (unsigned big = __ballot_sync(kFull, own && Ni > kLaneSumMax); big; big &= big - 1) {
-    const int i = __ffs(big) - 1;
-    const int o0 = ct->off[i], o1 = ct->off[i + 1];
-    for (int s = o0 + lane; s < o1; s += 32) sseg[s] = (uint8_t)i;
-  }
+  // the cell of slot sb + lane, for the 32 slots from sb (by the whole warp):
+  // the cells that start up to it, from the lanes' own offsets
+  const unsigned ne = __ballot_sync(kFull, own && Ni > 0);
+  if (own && Ni > 0) ct->ne[__popc(ne & ((1u << lane) - 1u))] = (uint8_t)lane;
+  const unsigned upto = 0xFFFFFFFFu >> (31 - lane);
+  const auto slot_cell = [&](int sb) -> int {
+    const bool has = own && Ni > 0;
+    const unsigned heads = __reduce_or_sync(kFull, has && offi > sb && offi < sb + 32 ? 1u << (offi - sb) : 0u);
+    const int before = __popc(__ballot_sync(kFull, has && offi <= sb));
+    return ct->ne[before - 1 + __popc(heads & upto)];
+  };
+  // instance-local index of the batch's cell c (Philox counter)
+  const auto kl_of = [&](int c) -> uint32_t {
+    if constexpr (ONE) return (uint32_t)(k0 + c);
+    else return (uint32_t)(k0 + c - a.P[ct->inst[c]].cell_off);
+  };
   cp_async_wait_all();
   __syncwarp();
   // ---- 1b. Bird's sub-cells (option): each cell's slots in a stable order
@@ -1739,38 +1745,38 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   const int nsub_i = own ? inst_params<ONE>(a, inst).nsub : 1;
   const unsigned subs = __ballot_sync(kFull, nsub_i > 1);
   if (subs) {
-    for (int s = lane; s < M; s += 32) {
-      const int c = sseg[s];
+    uint16_t* slot_sub = (uint16_t*)tags;
+    for (int sb = 0; sb < M; sb += 32) {
+      const int s = sb + lane, c = slot_cell(sb);
       int sub = 0;
-      if ((subs >> c) & 1u) {
+      if (s < M && ((subs >> c) & 1u)) {
         const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
         T x[3] = {0, 0, 0};
         const uint32_t o = sidx[s];
 #pragma unroll
         for (int d = 0; d < DIM; ++d) x[d] = ((const T*)a.Apos[d])[o];
-        sub = subcell_of<T, DIM>(P, ct->kl[c], x);
+        sub = subcell_of<T, DIM>(P, kl_of(c), x);
       }
-      stag[s] = sub;
+      if (s < M) slot_sub[s] = (uint16_t)sub;
     }
     __syncwarp();
     if (nsub_i > 1) {  // lane i: a counting sort of cell i's slots (stable)
-      uint16_t* so = ct->soff[lane];
+      uint16_t* so = soff[lane];
       for (int t = 0; t <= nsub_i; ++t) so[t] = 0;
-      for (int s = offi; s < offi + Ni; ++s) so[stag[s] + 1] += 1;
+      for (int s = offi; s < offi + Ni; ++s) so[slot_sub[s] + 1] += 1;
       for (int t = 0; t < nsub_i; ++t) so[t + 1] += so[t];
       uint32_t* tmp = (uint32_t*)svy;  // free until the gather
-      for (int s = offi; s < offi + Ni; ++s) tmp[offi + so[stag[s]]++] = sidx[s];
+      for (int s = offi; s < offi + Ni; ++s) tmp[offi + so[slot_sub[s]]++] = sidx[s];
       for (int t = nsub_i; t > 0; --t) so[t] = so[t - 1];
       so[0] = 0;
       for (int s = offi; s < offi + Ni; ++s) sidx[s] = tmp[s];
     }
     __syncwarp();
-  }
-  // the free flight reads the source indices from perm: store the sub-cell
-  // order there
-  if (subs) {
-    for (int s = lane; s < M; s += 32)
-      if ((subs >> sseg[s]) & 1u) a.perm[p0 + s] = sidx[s];
+    // the free flight reads the source indices from perm: store the sub-cell
+    // order there
+    if (nsub_i > 1)
+      for (int s = offi; s < offi + Ni; ++s) a.perm[p0 + s] = sidx[s];
+    __syncwarp();
   }
   // ---- 2. gather velocities (with the indices in the x-velocity array,
   // each lane reads slot s's index before it writes slot s's velocity);
@@ -1785,8 +1791,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       cp_async<sizeof(T)>(&svx[s], &Av0[o]);
       cp_async<sizeof(T)>(&svy[s], &Av1[o]);
       cp_async<sizeof(T)>(&svz[s], &Av2[o]);
-      stag[s] = 0x7FFFFFFF;
     }
+    for (int s = lane; s < ntag; s += 32) tags[s] = 0x7FFFFFFF;
     cp_async_wait_all();
   }
   __syncwarp();
@@ -1926,10 +1932,10 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     smaxT = (T)smax_k;
     bool settled = false;
     if constexpr (kMixed)
-      settled = cell_settled(Pi, (uint32_t)ct->kl[lane], Ni, sum_h, sum_h[3], vol_k, a.iLc, kc, smaxT, dt_k, dt_min_k,
+      settled = cell_settled(Pi, kl_of(lane), Ni, sum_h, sum_h[3], vol_k, a.iLc, kc, smaxT, dt_k, dt_min_k,
                              step, cm);
     if (!settled)
-      cell_math<T, A, !kMixed>(a, Pi, kc, (uint32_t)ct->kl[lane], Ni, m0, m1, m2, mS2, mS3x, mS3y, mS3z, vol_k,
+      cell_math<T, A, !kMixed>(a, Pi, kc, kl_of(lane), Ni, m0, m1, m2, mS2, mS3x, mS3y, mS3z, vol_k,
                                smaxT, dt_k, step, cm);
     ct->Pres[lane] = 0;
     if (cm.shk) {
@@ -2031,9 +2037,9 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       for (int k = 0; k < nround; ++k) {
         if (lane_ntc && k < (int)ncol) {
           const int N = Ni;
-          const NtcDraw<T> dr = ntc_draw((T)0, step, (uint32_t)ct->kl[lane], (uint32_t)k, Pi.key0, Pi.key1);
+          const NtcDraw<T> dr = ntc_draw((T)0, step, kl_of(lane), (uint32_t)k, Pi.key0, Pi.key1);
           int ci, cj;
-          select_pair(N, dr.u1, dr.u2, ct->soff[lane], nsub_i, &ci, &cj);
+          select_pair(N, dr.u1, dr.u2, soff[lane], nsub_i, &ci, &cj);
           ci += offi;
           cj += offi;
           const T ax = svx[ci], ay = svy[ci], az = svz[ci];
@@ -2056,7 +2062,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
             if (pass) {
               cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
               u4 = dr.u4();
-              u5 = ntc_u5(step, (uint32_t)ct->kl[lane], (uint32_t)k, Pi.key0, Pi.key1);
+              u5 = ntc_u5(step, kl_of(lane), (uint32_t)k, Pi.key0, Pi.key1);
             }
           }
           if (pass) {
@@ -2098,15 +2104,21 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       c = lo;
       const int N = ct->off[c + 1] - ct->off[c];
       const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-      dr = ntc_draw((T)0, step, (uint32_t)ct->kl[c], (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
-      select_pair(N, dr.u1, dr.u2, ct->soff[c], P.nsub, &ci, &cj);
+      dr = ntc_draw((T)0, step, kl_of(c), (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
+      select_pair(N, dr.u1, dr.u2, soff[c], P.nsub, &ci, &cj);
       ci += ct->off[c];
       cj += ct->off[c];
     }
     const int cnext = __shfl_down_sync(kFull, c, 1), cprev = __shfl_up_sync(kFull, c, 1);
     const bool seg_last = valid && (lane == 31 || cnext != c);
+    // the slots' entries in the folded tag table (ntag entries, slots below
+    // 2 ntag + 2): two slots that share one only wait for each other
+    const auto fold = [&](int s) {
+      s = s < ntag ? s : s - ntag;
+      return s < ntag ? s : s - ntag;
+    };
+    const int ti = fold(ci), tj = fold(cj);
     // the first lane of this lane's cell
-    const unsigned upto = 0xFFFFFFFFu >> (31 - lane);
     const int seg0 = 31 - __clz((int)(__ballot_sync(kFull, lane == 0 || c != cprev) & upto));
     const T coef = valid ? geo<T>(inst_params<ONE>(a, ct->inst[c])).sigc_coef : (T)0;
     const T ex = valid ? geo<T>(inst_params<ONE>(a, ct->inst[c])).sigc_exp : (T)0;
@@ -2122,23 +2134,23 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     // when it fails already against the prefix maximum of the evaluated
     // ones (the full maximum can only be larger, so it fails too: rejected,
     // nothing changes).  Accepted candidates of one pass share no particle,
-    // and every pass decides at least the first pending candidate of each
-    // cell, so the outcome is that of the one-by-one loop.
+    // and every pass decides at least the first pending candidate, so the
+    // outcome is that of the one-by-one loop.
     bool known = false;
     T ax = 0, ay = 0, az = 0, bx = 0, by = 0, bz = 0, cr = 0, sc = (T)-1;
     NtcTest tt = {-1.0, 0.0f, false};
     while (pending) {
       const bool mine = (pending >> lane) & 1u;
       if (mine) {
-        atomicMin(&stag[ci], lane);
-        atomicMin(&stag[cj], lane);
+        atomicMin(&tags[ti], lane);
+        atomicMin(&tags[tj], lane);
       }
       __syncwarp();
-      const bool ev = mine && stag[ci] == lane && stag[cj] == lane;
+      const bool ev = mine && tags[ti] == lane && tags[tj] == lane;
       __syncwarp();
       if (mine) {
-        stag[ci] = 0x7FFFFFFF;
-        stag[cj] = 0x7FFFFFFF;
+        tags[ti] = 0x7FFFFFFF;
+        tags[tj] = 0x7FFFFFFF;
       }
       if (ev && !known) {
         ax = svx[ci]; ay = svy[ci]; az = svz[ci];
@@ -2184,7 +2196,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
           const T g0 = ax - bx, g1 = ay - by, g2 = az - bz;
           cr = csqrt(g0 * g0 + g1 * g1 + g2 * g2);
           u4 = dr.u4();
-          u5 = ntc_u5(step, (uint32_t)ct->kl[c], (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
+          u5 = ntc_u5(step, kl_of(c), (uint32_t)(g - ct->coff[c]), P.key0, P.key1);
         }
         const T cchi = (T)2.0 * u4 - (T)1.0;
         const T schi = csqrt((T)1.0 - cchi * cchi);
@@ -2220,7 +2232,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     a.smax[kc] = (double)ct->smax[lane];
   }
   // ---- 6. Shakhov sub-step.  First the Bernoulli draw of every slot, with
-  // the resampled slots compacted into a list (stag is free after the DSMC
+  // the resampled slots compacted into a list (the tags' bytes, free after the DSMC
   // loop); then the acceptance-rejection loops as a lane pool: a lane that
   // finishes a particle takes the next one from the list, so the warp's
   // iterations follow the total number of attempts instead of the slowest
@@ -2228,29 +2240,29 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   // so the order of the work changes no result.
   if (__any_sync(kFull, shk)) {
     int nlist = 0;
+    uint16_t* list = (uint16_t*)tags;  // cell << 10 | slot (at most 1024 slots)
     for (int sb = 0; sb < M; sb += 32) {
-      const int s = sb + lane;
+      const int s = sb + lane, c = slot_cell(sb);
       bool res = false;
       if (s < M) {
-        const int c = sseg[s];
         const T Pres = ct->Pres[c];
         if (Pres > (T)0) {
           const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-          Uni<T> r(step, (uint32_t)ct->kl[c], (uint32_t)(s - ct->off[c]), kPurpShk << 24, P.key0, P.key1);
+          Uni<T> r(step, kl_of(c), (uint32_t)(s - ct->off[c]), kPurpShk << 24, P.key0, P.key1);
           res = r.get(0) < Pres;
         }
       }
       const unsigned bal = __ballot_sync(kFull, res);
       if (res) {
-        stag[nlist + __popc(bal & ((1u << lane) - 1u))] = s;
-        atomicAdd(&ct->nres[sseg[s]], 1);
+        list[nlist + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(c << 10 | s);
+        atomicAdd(&ct->nres[c], 1);
         if (a.resamp) a.resamp[p0 + s] = 1;
       }
       nlist += __popc(bal);
     }
     __syncwarp();
     if (nlist > 0) {
-      int s = lane < nlist ? stag[lane] : -1;
+      int s = lane < nlist ? list[lane] : -1;
       int next = 32, t = 0, c = 0, armax = 1;
       T RT = 0, s2RT = 0, Amax = 0, omp = 0, q0 = 0, q1 = 0, q2 = 0, kA = 0, iRT = 0;
       ShakhovFilter fl = {};
@@ -2259,9 +2271,10 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         s = slot;
         t = 0;
         if (s < 0) return;
-        c = sseg[s];
+        c = s >> 10;
+        s &= 1023;
         const InstParams& P = inst_params<ONE>(a, ct->inst[c]);
-        r = Uni<T>(step, (uint32_t)ct->kl[c], (uint32_t)(s - ct->off[c]), kPurpShk << 24, P.key0, P.key1);
+        r = Uni<T>(step, kl_of(c), (uint32_t)(s - ct->off[c]), kPurpShk << 24, P.key0, P.key1);
         armax = P.ar_max;
         RT = ct->RT[c];
         s2RT = ct->s2RT[c];
@@ -2297,7 +2310,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         const unsigned fin = __ballot_sync(kFull, done);
         if (done) {
           const int idx = next + __popc(fin & ((1u << lane) - 1u));
-          take(idx < nlist ? stag[idx] : -1);
+          take(idx < nlist ? list[idx] : -1);
         }
         next += __popc(fin);
       }
@@ -2337,7 +2350,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       });
       if (rown) {
         const double Tp = (double)r2[0] / (3.0 * Pi.R * (double)(Ni - 1));
-        ct->f[lane] = Tp > 0 ? (T)sqrt((double)TA / Tp) : (T)-1;
+        ct->q[0][lane] = Tp > 0 ? (T)sqrt((double)TA / Tp) : (T)-1;
         if constexpr (sizeof(A) == 8) {  // (T_p = 0: not rescaled, every velocity is U_p)
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
@@ -2348,10 +2361,10 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         }
       }
       __syncwarp();
-      for (int s = lane; s < M; s += 32) {
-        const int c = sseg[s];
-        if (!((rcells >> c) & 1u)) continue;
-        const T f = ct->f[c];
+      for (int sb = 0; sb < M; sb += 32) {
+        const int s = sb + lane, c = slot_cell(sb);
+        if (s >= M || !((rcells >> c) & 1u)) continue;
+        const T f = ct->q[0][c];
         if (!(f > (T)0)) continue;
         svx[s] = ct->U[0][c] + (svx[s] - ct->Up[0][c]) * f;
         svy[s] = ct->U[1][c] + (svy[s] - ct->Up[1][c]) * f;
@@ -2394,8 +2407,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         if (Sp > 0) {
           // f = sqrt(T / T_p), T_p = sum |c - U_p|^2 / (3 R (N - 1))
           const A f = sqrt(TA * (A)3.0 * (A)Pi.R * (A)(Ni - 1) / Sp);
-          ct->f[lane] = (T)f;
-          ct->fl[lane] = (T)(f - (A)(T)f);
+          ct->q[0][lane] = (T)f;
+          ct->q[1][lane] = (T)(f - (A)(T)f);
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             const A K = UA[d] - Upd[d] * f;
@@ -2406,7 +2419,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
             bsq[d] = f * f * Sii[d] + (A)Ni * UA[d] * UA[d];
           }
         } else {
-          ct->f[lane] = (T)-1;
+          ct->q[0][lane] = (T)-1;
 #pragma unroll
           for (int d = 0; d < 3; ++d) bsq[d] = Sii[d] + (A)Ni * Upd[d] * Upd[d];
         }
@@ -2415,14 +2428,14 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
       if (a.cons) {
         // record mode: the FP64 values of the rescaled velocities (before
         // they are rounded to FP32) summed in FP64, against the targets
-        const bool chk = rown && ct->f[lane] > (T)0;
+        const bool chk = rown && ct->q[0][lane] > (T)0;
         double r3[4];
         cell_sums<PlainSum<double>, 4>(lp, chk, offi, Ni, r3, [&](int s, int c, double* v, double* lo) {
           const T x[3] = {svx[s], svy[s], svz[s]};
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             float l;
-            const float h = affine_ff(x[d], ct->f[c], ct->fl[c], ct->Up[d][c], ct->Kl[d][c], &l);
+            const float h = affine_ff(x[d], ct->q[0][c], ct->q[1][c], ct->Up[d][c], ct->Kl[d][c], &l);
             v[d] = (double)h + (double)l;
             lo[d] = 0;
           }
@@ -2431,17 +2444,17 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
         });
         if (chk) record_conservation(a, kc, Ni, Pi, UA, TA, r3);
       }
-      for (int s = lane; s < M; s += 32) {
-        const int c = sseg[s];
-        if (!((rcells >> c) & 1u)) continue;
-        const T f = ct->f[c];
+      for (int sb = 0; sb < M; sb += 32) {
+        const int s = sb + lane, c = slot_cell(sb);
+        if (s >= M || !((rcells >> c) & 1u)) continue;
+        const T f = ct->q[0][c];
         if (!(f > (T)0)) continue;
         float l;
-        float h = affine_ff(svx[s], f, ct->fl[c], ct->Up[0][c], ct->Kl[0][c], &l);
+        float h = affine_ff(svx[s], f, ct->q[1][c], ct->Up[0][c], ct->Kl[0][c], &l);
         svx[s] = h + l;
-        h = affine_ff(svy[s], f, ct->fl[c], ct->Up[1][c], ct->Kl[1][c], &l);
+        h = affine_ff(svy[s], f, ct->q[1][c], ct->Up[1][c], ct->Kl[1][c], &l);
         svy[s] = h + l;
-        h = affine_ff(svz[s], f, ct->fl[c], ct->Up[2][c], ct->Kl[2][c], &l);
+        h = affine_ff(svz[s], f, ct->q[1][c], ct->Up[2][c], ct->Kl[2][c], &l);
         svz[s] = h + l;
       }
       __syncwarp();
@@ -2449,7 +2462,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     if constexpr (sizeof(T) == 8) {
       if (a.cons) {
         // record mode, FP64 mode: the rescaled velocities summed in FP64
-        const bool chk = rown && ct->f[lane] > (T)0;
+        const bool chk = rown && ct->q[0][lane] > (T)0;
         double r3[4];
         cell_sums<PlainSum<double>, 4>(lp, chk, offi, Ni, r3, [&](int s, int c, double* v, double* lo) {
           v[0] = svx[s];
@@ -2551,9 +2564,11 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cap = big ? a.big_cap : a.cap_small;
   if (big && warp != 0) return;
-  unsigned char* base = smem + (size_t)(big ? 0 : warp) * warp_stage_bytes<T, A>(cap);
+  const bool subs = a.subcells != 0;
+  unsigned char* base = smem + (size_t)(big ? 0 : warp) * warp_stage_bytes<T, A>(cap, subs);
   CellTab<T, A>* ct = (CellTab<T, A>*)base;
-  T* svx = (T*)(base + sizeof(CellTab<T, A>));
+  uint16_t(*soff)[kMaxSub + 1] = (uint16_t(*)[kMaxSub + 1])(base + sizeof(CellTab<T, A>));
+  T* svx = (T*)(base + sizeof(CellTab<T, A>) + (subs ? kSubBytes : 0));
   T* svy = svx + cap;
   T* svz = svy + cap;
   unsigned char* tail = (unsigned char*)(svz + cap);
@@ -2562,8 +2577,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1
     sidx = (uint32_t*)tail;
     tail += 4 * (size_t)cap;
   }
-  int* stag = (int*)tail;
-  uint8_t* sseg = (uint8_t*)(stag + cap);
+  int* tags = (int*)tail;
   // One call site of process_batch for both launches, so that every cell
   // runs through the same inlined code (identical rounding whichever launch
   // or batch takes it).  Main launch: batches from the plan's four class
@@ -2606,7 +2620,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1
       if ((int)(a.start[k0 + 1] - a.start[k0]) > kHugeCell) continue;  // k_collide_huge's cell
     }
     const long long t0 = clock64();
-    process_batch<T, A, DIM, ONE>(a, k0, G, ct, sidx, stag, sseg, svx, svy, svz);
+    process_batch<T, A, DIM, ONE>(a, k0, G, ct, sidx, tags, cap / 2, soff, svx, svy, svz);
     if (!big) {
       // the batch's cost steers the next step's plan (no effect on results):
       // its cycles per particle in units of cyc[2] (1/16 of the last step's

@@ -153,6 +153,7 @@ struct StepArgs {
   int cap_small;        // staging capacity per warp of the main launch
   double* surf;         // [elements][kSurfFields] wall tallies
   int one;              // a single instance: P0 is its parameter set
+  int subcells;         // an instance uses sub-cells
   // body-fitted O-grid instances (mesh = 1; all instances of a context
   // share the mesh kind): per-cell size L of Delta t_c and 1/L, faces
   // (state type, [NC][4][3]: outward unit normal, offset), nodes (state
@@ -193,9 +194,9 @@ struct InjectArgs {
 struct KernelSet {
   void (*collide)(int dim, const StepArgs& a, bool big, int grid, int warps, cudaStream_t s);
   void (*collide_huge)(int dim, const StepArgs& a, int grid, cudaStream_t s);
-  size_t (*collide_smem)(int warps, int cap);
+  bool (*collide_fits)(int warps, int cap);
   void (*flight)(int dim, const StepArgs& a, int nsm, cudaStream_t s);
-  int (*collide_blocks_per_sm)(int dim, int warps, int cap, bool one);
+  int (*collide_blocks_per_sm)(int dim, int warps, int cap, bool one, bool subcells);
   cudaError_t (*configure)();
   void (*inject)(int dim, const InjectArgs& a, int pass, cudaStream_t s);
   void (*moments)(const StepArgs& a, int64_t c0, int64_t c1, double* out, cudaStream_t s);

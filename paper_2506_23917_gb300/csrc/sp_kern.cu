@@ -20,10 +20,10 @@ using A = SP_KA;
 template <int DIM, bool ONE>
 void collide_dim1(const StepArgs& a, bool big, int grid, int warps, cudaStream_t s) {
   if (!big) {
-    const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(a.cap_small);
+    const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(a.cap_small, a.subcells != 0);
     k_collide<T, A, DIM, ONE><<<grid, 32 * warps, smem, s>>>(a, 0);
   } else {
-    const size_t smem = warp_stage_bytes<T, A>(a.big_cap);
+    const size_t smem = warp_stage_bytes<T, A>(a.big_cap, a.subcells != 0);
     k_collide<T, A, DIM, ONE><<<grid, 32, smem, s>>>(a, 1);
   }
 }
@@ -40,7 +40,17 @@ void collide(int dim, const StepArgs& a, bool big, int grid, int warps, cudaStre
   else collide_dim<3>(a, big, grid, warps, s);
 }
 
-size_t collide_smem(int warps, int cap) { return (size_t)warps * warp_stage_bytes<T, A>(cap); }
+// Whether sp_set_schedule takes a schedule: the limit it has always had, a
+// staging area of 17 (FP32) or 33 (FP64) bytes per particle and a table of
+// 4240 or 6928 bytes per warp within the block's shared memory (the present
+// layout is smaller).
+bool collide_fits(int warps, int cap) {
+  const size_t tab = sizeof(T) == 4 ? 4240 : 6928, per = sizeof(T) == 4 ? 17 : 33;
+  static_assert(sizeof(CellTab<T, A>) + kSubBytes + 4 <= (sizeof(T) == 4 ? 4240 : 6928) &&
+                    stage_bytes_per_particle<T>() <= (sizeof(T) == 4 ? 17 : 33),
+                "a schedule that was taken must fit");
+  return (size_t)warps * ((tab + per * (size_t)cap + 15) / 16 * 16) <= (size_t)kMaxDynSmem;
+}
 
 template <int DIM>
 void collide_huge_dim(const StepArgs& a, int grid, cudaStream_t s) {
@@ -180,8 +190,8 @@ int blocks_per_sm_dim(int warps, size_t smem, bool one) {
   return n;
 }
 
-int blocks_per_sm(int dim, int warps, int cap, bool one) {
-  const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(cap);
+int blocks_per_sm(int dim, int warps, int cap, bool one, bool subcells) {
+  const size_t smem = (size_t)warps * warp_stage_bytes<T, A>(cap, subcells);
   if (dim == 1) return blocks_per_sm_dim<1>(warps, smem, one);
   if (dim == 2) return blocks_per_sm_dim<2>(warps, smem, one);
   return blocks_per_sm_dim<3>(warps, smem, one);
@@ -189,7 +199,7 @@ int blocks_per_sm(int dim, int warps, int cap, bool one) {
 }  // namespace
 
 const KernelSet& SP_CAT(kernels, SP_TAG)() {
-  static const KernelSet k = {collide,  collide_huge, collide_smem, flight, blocks_per_sm, configure,
+  static const KernelSet k = {collide,  collide_huge, collide_fits, flight, blocks_per_sm, configure,
                               inject,   moments,      keys,             keys_mesh,       gather,
                               stage_in<double>,       stage_in<float>};
   return k;
