@@ -1027,11 +1027,13 @@ struct LanePart {
   int c, b, e;
   int own_parts, h0;
   uint16_t* scratch;  // [32] shared, for the FP64 sums
+  int home;           // an owner lane's cell above kLaneSumMax: home_lane
 };
 template <>
 struct LanePart<0> {
   static constexpr int split = 0;
   uint16_t* scratch;
+  int home;
 };
 
 // The lanes' parts of a batch of G cells (cells with Ni > kLaneSumMax: one
@@ -1041,6 +1043,7 @@ template <int split, class TabT>
 __device__ __forceinline__ LanePart<split> lane_parts(TabT* ct, int G, bool own, int offi, int Ni) {
   LanePart<split> lp;
   lp.scratch = ct->hpart;
+  lp.home = 0;
   if constexpr (split == 0) {
     return lp;
   } else {
@@ -1085,6 +1088,40 @@ __device__ __forceinline__ LanePart<split> lane_parts(TabT* ct, int G, bool own,
     }
     return lp;
   }
+}
+
+// The lane whose FP32 pair stands for the butterfly's sum of cell k (of
+// kLaneSumMax + 1 to kHomeCap particles; lane 0 above): the cell's place among
+// the cells of a partition of its chunk of 32 cells into runs of at most
+// kHomeCap particles and 32 lanes.  That is the batch partition of the
+// schedule that most FP32 flows are tuned to, whose sums are thus kept bit for
+// bit; taken from the actual batches, the lane -- and with it the last bits
+// of Shakhov cells -- would depend on the schedule.
+constexpr int kHomeCap = 864;
+__device__ __forceinline__ int home_lane(const uint32_t* start, int64_t NC, int64_t k, int split) {
+  const int lane = threadIdx.x & 31;
+  const int64_t c0 = k & ~(int64_t)31;
+  const int at = (int)(k - c0), nc = (int)(NC - c0 < 32 ? NC - c0 : 32);
+  uint32_t cum = lane < nc ? start[c0 + lane + 1] - start[c0 + lane] : 0u;
+  int lcum = lane < nc ? cell_lanes((int)(cum < 0x7FFFFFFFu ? cum : 0x7FFFFFFFu), split) : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, cum, o);
+    const int z = __shfl_up_sync(kFull, lcum, o);
+    if (lane >= o) {
+      cum += y;
+      lcum += z;
+    }
+  }
+  for (int kk = 0; kk <= at;) {
+    const uint32_t before = kk > 0 ? __shfl_sync(kFull, cum, kk - 1) : 0u;
+    const int lbefore = kk > 0 ? __shfl_sync(kFull, lcum, kk - 1) : 0;
+    const int G = __popc(__ballot_sync(kFull, lane >= kk && lane < nc && cum - before <= (uint32_t)kHomeCap &&
+                                                  lcum - lbefore <= 32));
+    if (at < kk + G) return at - kk;
+    kk += G > 0 ? G : 1;
+  }
+  return 0;
 }
 
 // Lanes that share the FP64 sum of a cell of n particles (a power of two,
@@ -1221,9 +1258,15 @@ __device__ __forceinline__ void cell_sums_acc(const LP& lp, bool own, int offi, 
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
       for (int k = 0; k < K; ++k) acc[k].combine(acc[k].shfl_xor(o));
-    if (lane == c)
+    // one lane's sum, fixed by the state (home_lane), whichever lane c the
+    // cell has in this batch: the lanes' error terms of the exact sums differ
+    // in their last bits
+    const int src = Acc::kExact ? __shfl_sync(kFull, lp.home, c) : 0;
 #pragma unroll
-      for (int k = 0; k < K; ++k) out[k] = acc[k];
+    for (int k = 0; k < K; ++k) {
+      const Acc y = acc[k].shfl_from(src);
+      if (lane == c) out[k] = y;
+    }
   }
   __syncwarp();
 }
@@ -1716,7 +1759,13 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   if (lane == 0) ct->off[G] = M;
   __syncwarp();
   // the lanes' parts of the per-cell sums (split cells: FP32 state only)
-  const auto lp = lane_parts<kSplitOf<T, DIM>>(ct, G, own, offi, Ni);
+  auto lp = lane_parts<kSplitOf<T, DIM>>(ct, G, own, offi, Ni);
+  if constexpr (Acc::kExact) {
+    for (unsigned b = __ballot_sync(kFull, own && Ni > kLaneSumMax && Ni <= kHomeCap); b; b &= b - 1) {
+      const int c = __ffs(b) - 1, h = home_lane(a.start, NC, k0 + c, kSplitOf<T, DIM>);
+      if (lane == c) lp.home = h;
+    }
+  }
   // ---- 1. source indices (in source order within each cell when the run is
   // reproducible: k_order) and cell of each slot
 #pragma unroll 4
