@@ -219,12 +219,97 @@ __device__ __forceinline__ void order_entries(uint32_t (&x)[R], uint32_t* p, int
   }
 }
 
-template <int R>
+// The same for entries that arrive in runs: both scatters write the entries
+// that one warp found for a cell in one window of 32 source indices (x >> 5)
+// side by side and ascending, so a cell is a sequence of such runs, and only
+// their order has to be found.  A cell of 40 holds about 12 runs, one of 600
+// about 50.  Each run's place is the summed length of the runs of smaller
+// windows (a loop over the runs, each lane for up to Q of them); every entry
+// then moves with its run.  Up to 32 Q runs; false (nothing done) above.
+// sh: the warp's shared memory, 64 Q + 2 R words.  40-entry cells: about 95
+// instructions and 17 shuffles instead of 135 and 34; 600: 0.9 instructions
+// per entry instead of 4.5.
+template <int R, int Q>
+__device__ __forceinline__ bool order_runs(const uint32_t (&x)[R], uint32_t* p, int n, int lane, uint32_t* sh) {
+  uint32_t *rkey = sh, *rpos = sh + 32 * Q, *rmask = sh + 64 * Q, *rbase = rmask + R;
+  const unsigned le = 0xFFFFFFFFu >> (31 - lane);
+  int H = 0;
+  uint32_t prev = 0xFFFFFFFFu;  // the last entry of the row before
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    uint32_t before = __shfl_up_sync(0xFFFFFFFFu, x[i], 1);
+    if (lane == 0) before = prev;
+    const int t = 32 * i + lane;
+    const bool head = t < n && (t == 0 || (before >> 5) != (x[i] >> 5));
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, head);
+    const int q = H + __popc(m & le) - 1;
+    if (head && q < 32 * Q) {
+      rkey[q] = x[i] >> 5;
+      rpos[q] = (uint32_t)t;
+    }
+    if (lane == 0) {
+      rmask[i] = m;
+      rbase[i] = (uint32_t)H;
+    }
+    H += __popc(m);
+    if (R > 1) prev = __shfl_sync(0xFFFFFFFFu, x[i], 31);
+  }
+  __syncwarp();
+  if (H > 32 * Q) {
+    __syncwarp();
+    return false;
+  }
+  uint32_t key[Q];
+  int pos[Q], place[Q];
+#pragma unroll
+  for (int u = 0; u < Q; ++u) {
+    const int q = 32 * u + lane;
+    pos[u] = q < H ? (int)rpos[q] : n;
+    const int next = q + 1 < H ? (int)rpos[q + 1] : n;
+    key[u] = q < H ? rkey[q] << 5 | (uint32_t)(next - pos[u] - 1) : 0xFFFFFFFFu;  // (a run holds at most 32)
+    place[u] = 0;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < Q; ++u) rkey[32 * u + lane] = key[u];
+  __syncwarp();
+#pragma unroll 4
+  for (int j = 0; j < H; ++j) {
+    const uint32_t k = rkey[j];
+    const int len = (int)(k & 31u) + 1;
+#pragma unroll
+    for (int u = 0; u < Q; ++u) place[u] += k < key[u] ? len : 0;
+  }
+  bool moved = false;
+#pragma unroll
+  for (int u = 0; u < Q; ++u) {
+    const int q = 32 * u + lane;
+    if (q < H) {
+      rpos[q] = (uint32_t)(place[u] - pos[u]);  // how far the run moves
+      moved = moved || place[u] != pos[u];
+    }
+  }
+  __syncwarp();
+  if (__any_sync(0xFFFFFFFFu, moved)) {
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int t = 32 * i + lane;
+      if (t < n) {
+        const int q = (int)rbase[i] + __popc(rmask[i] & le) - 1;
+        p[t + (int)rpos[q]] = x[i];
+      }
+    }
+  }
+  __syncwarp();
+  return true;
+}
+
+template <int R, int Q>
 __device__ __forceinline__ void order_cell(uint32_t* p, int n, int lane, uint32_t* sh) {
   uint32_t x[R];
 #pragma unroll
   for (int i = 0; i < R; ++i) x[i] = 32 * i + lane < n ? p[32 * i + lane] : 0xFFFFFFFFu;
-  order_entries<R>(x, p, n, lane, sh);
+  if (!order_runs<R, Q>(x, p, n, lane, sh)) order_entries<R>(x, p, n, lane, sh);
 }
 
 // A cell of n <= 8 * 32 R entries by the whole block: warp w sorts entries
@@ -282,7 +367,9 @@ __device__ __forceinline__ void order_big_cell(uint32_t* g, int64_t n, uint32_t*
 constexpr int kOrderCells = 4;
 __global__ void __launch_bounds__(kOrderThreads, 6) k_order_small(const uint32_t* start, int64_t ncells,
                                                                   uint32_t* perm) {
+  __shared__ uint32_t sh[kOrderWarps][72];
   const int lane = threadIdx.x & 31;
+  uint32_t* ws = sh[threadIdx.x >> 5];
   const int64_t nw = (int64_t)gridDim.x * kOrderWarps;
   for (int64_t c0 = ((int64_t)blockIdx.x * kOrderWarps + (threadIdx.x >> 5)) * kOrderCells; c0 < ncells;
        c0 += nw * kOrderCells) {
@@ -304,9 +391,9 @@ __global__ void __launch_bounds__(kOrderThreads, 6) k_order_small(const uint32_t
         uint32_t y[1] = {x[j][0]};
         order_entries<1>(y, perm + s0, (int)n, lane, nullptr);
       } else if (n <= 64) {
-        order_entries<2>(x[j], perm + s0, (int)n, lane, nullptr);
+        if (!order_runs<2, 1>(x[j], perm + s0, (int)n, lane, ws)) order_entries<2>(x[j], perm + s0, (int)n, lane, nullptr);
       } else {
-        order_cell<4>(perm + s0, (int)n, lane, nullptr);
+        order_cell<4, 1>(perm + s0, (int)n, lane, ws);
       }
     }
   }
@@ -331,9 +418,9 @@ __global__ void __launch_bounds__(kOrderThreads, 4) k_order_large(const uint32_t
         const int src = __ffs(todo) - 1;
         uint32_t* p = perm + __shfl_sync(0xFFFFFFFFu, s0, src);
         const int m = (int)__shfl_sync(0xFFFFFFFFu, n, src);
-        if (m <= 256) order_cell<8>(p, m, lane, ws);
-        else if (m <= 512) order_cell<16>(p, m, lane, ws);
-        else order_cell<32>(p, m, lane, ws);
+        if (m <= 256) order_cell<8, 2>(p, m, lane, ws);
+        else if (m <= 512) order_cell<16, 2>(p, m, lane, ws);
+        else order_cell<32, 4>(p, m, lane, ws);
       }
     }
   } else {
