@@ -72,7 +72,8 @@ struct sp_ctx {
   unsigned long long* dt_min = nullptr;
   uint32_t *step_d = nullptr, *Mcur = nullptr, *Mtot = nullptr;
   unsigned long long* err = nullptr;
-  unsigned long long* herr = nullptr;  // page-locked copy of err (check_errors)
+  unsigned long long* herr = nullptr;  // page-locked copy of err (check_errors); [kNumErr]: upload's status
+  unsigned long long* herr_dev = nullptr;  // its device address
   GhostCell* ghosts = nullptr;
   int64_t n_ghost = 0;
   uint32_t *gcount = nullptr, *goff = nullptr, *gscan_part = nullptr;
@@ -83,21 +84,19 @@ struct sp_ctx {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaGraphExec_t pgraph[2] = {nullptr, nullptr};  // the same steps with timing events
   cudaEvent_t pev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  bool graph_ok = false;
   cudaStream_t side = nullptr;       // capture-time branches of the step graph (injection,
   cudaStream_t side2 = nullptr;      // big-cell launch, huge-cell launch)
   cudaStream_t side3 = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr, fork2_ev = nullptr, join2_ev = nullptr;
   cudaEvent_t fork3_ev = nullptr, join3_ev = nullptr;
+  cudaEvent_t pos_ev = nullptr, idx_ev = nullptr;  // upload: positions copied, cells indexed
+  bool direct = false;  // the last particles went straight into the state buffers
   int launches = 0;
   std::vector<double*> dstage;    // per instance: FP64 [dim][n] then [3][n], device
   std::vector<int64_t> stage_n, stage_cap;
   std::vector<int> stage_f32;     // per instance: the staged data is FP32
   uint32_t* part_inst = nullptr;  // [cap] instance of each uploaded particle
   std::vector<uint32_t> prev_start;  // [NC+1] of the state before the last step (record mode)
-  std::vector<unsigned long long> hinf, hmin;  // host mirrors used by upload()
-  std::vector<double> hdt;
-  uint32_t hM = 0;
   // body-fitted O-grid instances (all instances share the mesh kind)
   int mesh = 0;
   bool subcells = false;  // an instance uses sub-cells
@@ -604,46 +603,44 @@ void destroy_graphs(sp_ctx* c) {
       c->pgraph[i] = nullptr;
     }
   }
-  c->graph_ok = false;
 }
 
-sp_status build_graphs(sp_ctx* c) {
-  destroy_graphs(c);
-  if (!c->side) {
-    CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
-    CK(cudaStreamCreateWithFlags(&c->side2, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&c->fork2_ev, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&c->join2_ev, cudaEventDisableTiming));
-    CK(cudaStreamCreateWithFlags(&c->side3, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&c->fork3_ev, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&c->join3_ev, cudaEventDisableTiming));
-    for (int k = 0; k < 5; ++k) CK(cudaEventCreate(&c->pev[k]));
-  }
-  // per parity: the step graph, and the same graph with timing events at
-  // the kernel groups' boundaries (sp_step_profiled)
-  for (int prof = 0; prof < 2; ++prof)
-    for (int par = 0; par < 2; ++par) {
-      cudaStream_t cs;
-      CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-      cudaStream_t saved = c->stream;
-      c->stream = cs;
-      cudaGraph_t g;
-      cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-      if (e == cudaSuccess) {
-        const int n = enqueue_step(c, par, prof ? c->pev : nullptr);
-        if (!prof) c->launches = n;
-        e = cudaStreamEndCapture(cs, &g);
-      }
-      c->stream = saved;
-      cudaStreamDestroy(cs);
-      CK(e);
-      e = cudaGraphInstantiate(prof ? &c->pgraph[par] : &c->graph[par], g, 0);
-      cudaGraphDestroy(g);
-      CK(e);
+sp_status make_streams(sp_ctx* c) {
+  if (c->side) return SP_OK;
+  for (cudaStream_t* t : {&c->side, &c->side2, &c->side3}) CK(cudaStreamCreateWithFlags(t, cudaStreamNonBlocking));
+  for (cudaEvent_t* e : {&c->fork_ev, &c->join_ev, &c->fork2_ev, &c->join2_ev, &c->fork3_ev, &c->join3_ev, &c->pos_ev,
+                         &c->idx_ev})
+    CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  for (int k = 0; k < 5; ++k) CK(cudaEventCreate(&c->pev[k]));
+  return SP_OK;
+}
+
+// Capture the step graphs of both buffer parities; prof: the copies with
+// timing events at the kernel groups' boundaries (built when first wanted).
+sp_status build_graphs(sp_ctx* c, bool prof = false) {
+  const sp_status st = make_streams(c);
+  if (st != SP_OK) return st;
+  cudaGraphExec_t* out = prof ? c->pgraph : c->graph;
+  for (int par = 0; par < 2; ++par) {
+    if (out[par]) continue;
+    cudaStream_t cs;
+    CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    cudaStream_t saved = c->stream;
+    c->stream = cs;
+    cudaGraph_t g;
+    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      const int n = enqueue_step(c, par, prof ? c->pev : nullptr);
+      c->launches = n;
+      e = cudaStreamEndCapture(cs, &g);
     }
-  c->graph_ok = true;
+    c->stream = saved;
+    cudaStreamDestroy(cs);
+    CK(e);
+    e = cudaGraphInstantiate(&out[par], g, 0);
+    cudaGraphDestroy(g);
+    CK(e);
+  }
   return SP_OK;
 }
 
@@ -664,59 +661,75 @@ sp_status upload(sp_ctx* c) {
   for (int i = 0; i < c->n_inst; ++i) M += c->stage_n[i];
   if (M > c->cap) return SP_ERR_CAPACITY;
   const int dim = c->dim;
-  int64_t off = 0;
-  for (int i = 0; i < c->n_inst; ++i) {
-    const int64_t n = c->stage_n[i];
-    if (n > 0) {
-      const double* sp = c->dstage[i];
-      const float* sf = (const float*)c->dstage[i];
-      if (c->stage_f32[i])
-        c->K->stage_in32(dim, sf, sf + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst,
-                         (uint32_t)i, c->stream);
-      else
-        c->K->stage_in(dim, sp, sp + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst,
-                       (uint32_t)i, c->stream);
+  cudaStream_t ix = c->stream;  // where the cells are indexed
+  if (c->direct) {
+    // the positions were copied first: index the cells while the velocities
+    // are on their way
+    ix = c->side;
+    CK(cudaStreamWaitEvent(ix, c->pos_ev, 0));
+  } else {
+    int64_t off = 0;
+    for (int i = 0; i < c->n_inst; ++i) {
+      const int64_t n = c->stage_n[i];
+      if (n > 0) {
+        const double* sp = c->dstage[i];
+        const float* sf = (const float*)c->dstage[i];
+        if (c->stage_f32[i])
+          c->K->stage_in32(dim, sf, sf + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst, (uint32_t)i, ix);
+        else
+          c->K->stage_in(dim, sp, sp + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst, (uint32_t)i, ix);
+      }
+      off += n;
     }
-    off += n;
   }
-  CK(cudaMemsetAsync(c->count, 0, sizeof(uint32_t) * c->NC, c->stream));
+  CK(cudaMemsetAsync(c->count, 0, sizeof(uint32_t) * c->NC, ix));
   const void* P3[3] = {c->pos[c->cur][0], c->pos[c->cur][1], c->pos[c->cur][2]};
   if (c->mesh)
-    c->K->keys_mesh(P3, M, c->part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key[c->cur], c->count, c->stream);
+    c->K->keys_mesh(P3, M, c->part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key[c->cur], c->count, ix);
   else
-    c->K->keys(dim, P3, M, c->part_inst, c->dP, c->key[c->cur], c->count, c->stream);
-  launch_scan(c->count, c->start, c->NC, c->scan_part, c->stream);
-  c->hM = (uint32_t)M;
-  CK(cudaMemcpyAsync(c->Mtot, &c->hM, 4, cudaMemcpyHostToDevice, c->stream));
+    c->K->keys(dim, P3, M, c->part_inst, c->dP, c->key[c->cur], c->count, ix);
+  launch_scan(c->count, c->start, c->NC, c->scan_part, ix);
   // the state holds the located particles only: an O-grid drops those
   // outside the mesh (sentinel keys), so its size is start[NC], not M
-  CK(cudaMemcpyAsync(c->Mcur, c->start + c->NC, 4, cudaMemcpyDeviceToDevice, c->stream));
-  launch_scatter(c->key[c->cur], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream);
+  launch_counts((uint32_t)M, c->start + c->NC, c->Mtot, c->Mcur, ix);
+  launch_scatter(c->key[c->cur], c->start, c->count, c->perm, c->Mtot, c->cap, ix);
   // the scatter's atomics leave each cell's order arbitrary: reproducible
   // runs restore the source order, so that the moments below (and the first
   // step's Delta t) sum each cell in the same order on every run
-  if (c->stable) launch_order_cells(c->start, c->NC, c->perm, c->stream);
-  // Delta t from the moments of this state
-  for (int i = 0; i < c->n_inst; ++i) c->hinf[i] = 0x7FF0000000000000ull;
-  CK(cudaMemcpyAsync(c->dt_min, c->hinf.data(), 8 * c->n_inst, cudaMemcpyHostToDevice, c->stream));
-  StepArgs a = make_step_args(c, c->cur);
-  c->K->moments(a, 0, c->NC, nullptr, c->stream);
-  CK(cudaMemcpyAsync(c->hmin.data(), c->dt_min, 8 * c->n_inst, cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  for (int i = 0; i < c->n_inst; ++i) {
-    if (c->hP[i].dt_fixed > 0) c->hdt[i] = c->hP[i].dt_fixed;
-    else if (c->hmin[i] != 0x7FF0000000000000ull) {
-      double v;
-      memcpy(&v, &c->hmin[i], 8);
-      c->hdt[i] = c->hP[i].cfl * v;
-    } else {
-      return SP_ERR_ARG;  // no cell with two particles and no fixed step
-    }
+  if (c->stable) launch_order_cells(c->start, c->NC, c->perm, ix);
+  if (c->direct) {
+    CK(cudaEventRecord(c->idx_ev, ix));
+    CK(cudaStreamWaitEvent(c->stream, c->idx_ev, 0));
   }
-  CK(cudaMemcpyAsync(c->dt_cur, c->hdt.data(), 8 * c->n_inst, cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemcpyAsync(c->dt_min, c->hinf.data(), 8 * c->n_inst, cudaMemcpyHostToDevice, c->stream));
+  // Delta t from the moments of this state
+  const StepArgs a = make_step_args(c, c->cur);
+  c->K->moments(a, 0, c->NC, nullptr, c->stream);
+  volatile unsigned long long* bad = c->herr + kNumErr;
+  *bad = 0;
+  launch_first_dt(c->dP, c->n_inst, c->dt_cur, c->dt_min, c->herr_dev + kNumErr, c->stream);
+  CK(cudaStreamSynchronize(c->stream));
+  if (*bad) return SP_ERR_ARG;  // no cell with two particles and no fixed step
   c->uploaded = true;
   c->dirty = false;
+  return SP_OK;
+}
+
+// A single instance's particles in the context's own type: straight into the
+// current state buffers (nothing reads the old state from here on: every
+// entry point that needs particles uploads first), positions ahead of the
+// velocities, so that upload() can index them meanwhile.
+template <class T>
+sp_status set_direct(sp_ctx* c, const T* pos, const T* vel, int64_t n) {
+  const sp_status st = make_streams(c);
+  if (st != SP_OK) return st;
+  c->dirty = true;
+  c->direct = true;
+  c->stage_n[0] = n;
+  for (int d = 0; d < c->dim && n > 0; ++d)
+    CK(cudaMemcpyAsync(c->pos[c->cur][d], pos + d * n, sizeof(T) * n, cudaMemcpyHostToDevice, c->stream));
+  CK(cudaEventRecord(c->pos_ev, c->stream));
+  for (int d = 0; d < 3 && n > 0; ++d)
+    CK(cudaMemcpyAsync(c->vel[c->cur][d], vel + d * n, sizeof(T) * n, cudaMemcpyHostToDevice, c->stream));
   return SP_OK;
 }
 
@@ -801,9 +814,6 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
   c->stage_n.assign(n_instances, 0);
   c->stage_cap.assign(n_instances, 0);
   c->stage_f32.assign(n_instances, 0);
-  c->hinf.assign(n_instances, 0x7FF0000000000000ull);
-  c->hmin.assign(n_instances, 0);
-  c->hdt.assign(n_instances, 0.0);
   // body-fitted O-grid instances: every instance of a context has the same
   // mesh kind (one kernel variant per launch)
   c->mesh = cfgs[0].mesh;
@@ -837,7 +847,7 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
         CK(dalloc(&c->vel[b][d], cap * c->tsize));
       }
     for (int b = 0; b < 2; ++b) CK(dalloc(&c->key[b], 4 * cap));
-    CK(dalloc(&c->part_inst, 4 * cap));
+    if (n_instances > 1) CK(dalloc(&c->part_inst, 4 * cap));
     CK(dalloc(&c->perm, 4 * cap));
     CK(dalloc(&c->count, 4 * NC));
     CK(dalloc(&c->start, 4 * (NC + 1)));
@@ -866,7 +876,8 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
     CK(dalloc(&c->Mcur, 4));
     CK(dalloc(&c->Mtot, 4));
     CK(dalloc(&c->err, 8 * kNumErr));
-    CK(cudaHostAlloc((void**)&c->herr, 8 * kNumErr, cudaHostAllocDefault));
+    CK(cudaHostAlloc((void**)&c->herr, 8 * (kNumErr + 1), cudaHostAllocMapped));
+    CK(cudaHostGetDevicePointer((void**)&c->herr_dev, c->herr, 0));
     CK(dalloc(&c->ghosts, sizeof(GhostCell) * std::max<int64_t>(c->n_ghost, 1)));
     CK(dalloc(&c->gcount, 4 * std::max<int64_t>(c->n_ghost, 1)));
     CK(dalloc(&c->goff, 4 * (std::max<int64_t>(c->n_ghost, 1) + 1)));
@@ -938,6 +949,8 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
     CK(cudaMemsetAsync(c->cost, 0, std::max<int64_t>(c->NC, 1), s));
     CK(cudaMemsetAsync(c->cyc, 0, 16, s));
     CK(cudaMemsetAsync(c->cyc + 2, 0xFF, 8, s));
+    const std::vector<unsigned long long> inf(n_instances, 0x7FF0000000000000ull);
+    CK(cudaMemcpyAsync(c->dt_min, inf.data(), 8 * n_instances, cudaMemcpyHostToDevice, s));
     int dev = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -958,6 +971,7 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
 sp_status sp_set_particles(sp_ctx* c, int inst, const double* pos, const double* vel, int64_t n) {
   if (!c || inst < 0 || inst >= c->n_inst || n < 0 || (n > 0 && (!pos || !vel))) return SP_ERR_ARG;
   if (n > c->cap) return SP_ERR_CAPACITY;
+  if (c->n_inst == 1 && c->tsize == 8) return set_direct(c, pos, vel, n);
   const int64_t need = (int64_t)(c->dim + 3) * n;
   if (need > c->stage_cap[inst]) {
     CK(cudaStreamSynchronize(c->stream));
@@ -972,6 +986,7 @@ sp_status sp_set_particles(sp_ctx* c, int inst, const double* pos, const double*
   }
   c->stage_n[inst] = n;
   c->stage_f32[inst] = 0;
+  c->direct = false;
   c->dirty = true;
   return SP_OK;
 }
@@ -979,6 +994,7 @@ sp_status sp_set_particles(sp_ctx* c, int inst, const double* pos, const double*
 sp_status sp_set_particles_f32(sp_ctx* c, int inst, const float* pos, const float* vel, int64_t n) {
   if (!c || inst < 0 || inst >= c->n_inst || n < 0 || (n > 0 && (!pos || !vel))) return SP_ERR_ARG;
   if (n > c->cap) return SP_ERR_CAPACITY;
+  if (c->n_inst == 1 && c->tsize == 4) return set_direct(c, pos, vel, n);
   const int64_t need = (int64_t)(c->dim + 3) * n;  // floats; the staging area counts doubles
   if ((need + 1) / 2 > c->stage_cap[inst]) {
     CK(cudaStreamSynchronize(c->stream));
@@ -994,6 +1010,7 @@ sp_status sp_set_particles_f32(sp_ctx* c, int inst, const float* pos, const floa
   }
   c->stage_n[inst] = n;
   c->stage_f32[inst] = 1;
+  c->direct = false;
   c->dirty = true;
   return SP_OK;
 }
@@ -1017,7 +1034,7 @@ sp_status sp_step(sp_ctx* c, int n_steps) {
   if (!c || n_steps < 0) return SP_ERR_ARG;
   sp_status s = ensure_ready(c);
   if (s != SP_OK) return s;
-  if (!c->graph_ok) {
+  if (!c->graph[1]) {
     s = build_graphs(c);
     if (s != SP_OK) return s;
   }
@@ -1040,8 +1057,8 @@ sp_status sp_step_profiled(sp_ctx* c, int n_steps, double* ms, int n_slots) {
   if (!c || n_steps < 0 || !ms || n_slots < 1) return SP_ERR_ARG;
   sp_status s = ensure_ready(c);
   if (s != SP_OK) return s;
-  if (!c->graph_ok) {
-    s = build_graphs(c);
+  if (!c->pgraph[1]) {
+    s = build_graphs(c, true);
     if (s != SP_OK) return s;
   }
   double acc[4] = {0, 0, 0, 0};
@@ -1096,7 +1113,8 @@ sp_status sp_autotune(sp_ctx* c, int steps_per_trial, int* cap_out, int* warps_o
   // changes with the schedule, and the cost bytes of the old one are stale)
   auto trial = [&](int ci, int wi, float* tot) -> sp_status {
     *tot = 0;
-    sp_status bs = build_graphs(c);
+    destroy_graphs(c);
+    sp_status bs = build_graphs(c, true);
     if (bs != SP_OK) return bs;
     for (int it = 0; it <= steps_per_trial; ++it) {
       CK(cudaGraphLaunch(c->pgraph[c->cur], c->stream));
@@ -1170,7 +1188,7 @@ sp_status sp_sync(sp_ctx* c) {
 
 int sp_launches_per_step(sp_ctx* c) {
   if (!c) return 0;
-  if (!c->graph_ok && c->uploaded) build_graphs(c);
+  if (!c->graph[1] && c->uploaded) build_graphs(c);
   return c->launches;
 }
 
@@ -1421,18 +1439,11 @@ sp_status sp_free(sp_ctx* c) {
   if (!c) return SP_ERR_ARG;
   cudaStreamSynchronize(c->stream);
   destroy_graphs(c);
-  if (c->side) {
-    cudaStreamDestroy(c->side);
-    cudaEventDestroy(c->fork_ev);
-    cudaEventDestroy(c->join_ev);
-    cudaStreamDestroy(c->side2);
-    cudaEventDestroy(c->fork2_ev);
-    cudaEventDestroy(c->join2_ev);
-    cudaStreamDestroy(c->side3);
-    cudaEventDestroy(c->fork3_ev);
-    cudaEventDestroy(c->join3_ev);
-    for (int k = 0; k < 5; ++k) cudaEventDestroy(c->pev[k]);
-  }
+  for (cudaStream_t t : {c->side, c->side2, c->side3})
+    if (t) cudaStreamDestroy(t);
+  for (cudaEvent_t e : {c->fork_ev, c->join_ev, c->fork2_ev, c->join2_ev, c->fork3_ev, c->join3_ev, c->pos_ev, c->idx_ev,
+                        c->pev[0], c->pev[1], c->pev[2], c->pev[3], c->pev[4]})
+    if (e) cudaEventDestroy(e);
   for (int b = 0; b < 2; ++b)
     for (int d = 0; d < 3; ++d) {
       cudaFree(c->pos[b][d]);

@@ -305,7 +305,32 @@ __global__ void k_mean_fields(const double* samp, int64_t NC, const double* vol,
   out[SP_F_ratio * nc + i] = ratio;
 }
 
+__global__ void k_counts(uint32_t M, const uint32_t* kept, uint32_t* Mtot, uint32_t* Mcur) {
+  *Mtot = M;
+  *Mcur = *kept;
+}
+
+__global__ void k_first_dt(const InstParams* P, int n_inst, double* dt_cur, unsigned long long* dt_min,
+                           unsigned long long* bad) {
+  const unsigned long long inf = 0x7FF0000000000000ull;
+  for (int i = threadIdx.x; i < n_inst; i += blockDim.x) {
+    if (P[i].dt_fixed > 0) dt_cur[i] = P[i].dt_fixed;
+    else if (dt_min[i] != inf) dt_cur[i] = P[i].cfl * __longlong_as_double((long long)dt_min[i]);
+    else *bad = 1ull;
+    dt_min[i] = inf;
+  }
+}
+
 }  // namespace
+
+void launch_counts(uint32_t M, const uint32_t* kept, uint32_t* Mtot, uint32_t* Mcur, cudaStream_t s) {
+  k_counts<<<1, 1, 0, s>>>(M, kept, Mtot, Mcur);
+}
+
+void launch_first_dt(const InstParams* P, int n_inst, double* dt_cur, unsigned long long* dt_min,
+                     unsigned long long* bad, cudaStream_t s) {
+  k_first_dt<<<1, 256, 0, s>>>(P, n_inst, dt_cur, dt_min, bad);
+}
 
 void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64_t c0, int64_t nc, double nsamp,
                         double Fn, double R, double* out, cudaStream_t s) {

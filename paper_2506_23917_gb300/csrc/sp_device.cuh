@@ -464,8 +464,8 @@ __device__ __forceinline__ bool flight_clear(const InstParams& P, const double* 
   }
   return ok;
 }
-// The cell of a point flight_clear has found inside the box: the FP32
-// coordinate decides unless it comes within 1e-6 of the span of a cell face.
+// cell_of for an FP64 state: the FP32 coordinate decides where it lies in the
+// grid and not within 1e-6 of the box's magnitude of a cell face.
 template <int DIM>
 __device__ __forceinline__ uint32_t cell_of_clear(const InstParams& P, const double* x) {
   const Geo<float>& G = P.g32;
@@ -3574,7 +3574,7 @@ __global__ void k_keys_mesh(const T* x0, const T* x1, int64_t M, const uint32_t*
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t k = kSentinel;
   if (i < M) {
-    const InstParams& P = Ps[part_inst[i]];
+    const InstParams& P = Ps[part_inst ? part_inst[i] : 0u];
     const T x[2] = {x0[i], x1[i]};
     const int64_t kl = mesh_locate<T>(P, mface, mnode, mrad, x);
     if (kl >= 0) k = (uint32_t)(P.cell_off + kl);
@@ -3587,7 +3587,7 @@ __global__ void k_keys_mesh(const T* x0, const T* x1, int64_t M, const uint32_t*
 // Observability / initialisation kernels
 // ---------------------------------------------------------------------------
 // Moments of the current state for cells [c0, c1), in the cells' current
-// slot order, in two kernels.  k_moment_sums: a half-warp (16 lanes) per
+// slot order, in two kernels.  k_moment_sums: kMomentLanes lanes per
 // cell; lanes stride over the cell's slots, a butterfly combines them, and
 // the first lane writes the cell's sums to sums[7][nc]: sum c (3), then
 // sum |C|^2 and, when the fields are wanted (kQ), sum |C|^2 C (3) about
@@ -3602,36 +3602,42 @@ __global__ void k_keys_mesh(const T* x0, const T* x1, int64_t M, const uint32_t*
 // scalars (U, n, T, q, tau, dt_c, the split ratio) from them on full warps,
 // and writes the fields to out [12][nc] or, with out == nullptr, takes the
 // minimum dt_c into dt_min (a warp minimum, then one atomic per warp).
+// Lanes per cell: 16 with an FP32 state; 4 with an FP64 state, where the
+// butterfly's additions hold the FP64 pipe as long as the terms' (2 M
+// particles, 30 per cell: 221 -> 118 us with the heat flux).
+template <class T>
+constexpr int kMomentLanes = sizeof(T) == 8 ? 4 : 16;
+
 template <class T, class A, bool kQ>
 __global__ void k_moment_sums(StepArgs a, int64_t c0, int64_t c1, double* sums) {
   using Acc = CellAcc<T, A>;
   constexpr bool kMixed = mixed_prec<T, A>();
   constexpr bool kPair = sizeof(T) == 4;
-  // a half-warp per cell (16 lanes, two cells per warp)
-  const int lane = threadIdx.x & 15;
-  const int64_t nh = (int64_t)gridDim.x * (blockDim.x >> 4);
+  constexpr int L = kMomentLanes<T>, W = 32 / L;  // lanes per cell, cells per warp
+  const int lane = threadIdx.x & (L - 1);
+  const int64_t nh = (int64_t)gridDim.x * (blockDim.x / L);
   const int64_t nc = c1 - c0;
   const T* Av0 = (const T*)a.Avel[0];
   const T* Av1 = (const T*)a.Avel[1];
   const T* Av2 = (const T*)a.Avel[2];
-  // the same trip count for both halves of a warp (the shuffles need all lanes)
-  const int64_t h0 = (int64_t)blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4);
-  for (int64_t kb = c0 + (h0 & ~(int64_t)1); kb < c1; kb += nh) {
-    const int64_t k = kb + (h0 & 1);
+  // the same trip count for all cells of a warp (the shuffles need all lanes)
+  const int64_t h0 = (int64_t)blockIdx.x * (blockDim.x / L) + threadIdx.x / L;
+  for (int64_t kb = c0 + (h0 & ~(int64_t)(W - 1)); kb < c1; kb += nh) {
+    const int64_t k = kb + (h0 & (W - 1));
     const bool valid = k < c1;
     const uint32_t s0 = valid ? a.start[k] : 0u;
     const int N = valid ? (int)(a.start[k + 1] - s0) : 0;
     Acc sx[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) sx[d].init();
-    for (int s = lane; s < N; s += 16) {
+    for (int s = lane; s < N; s += L) {
       const uint32_t o = a.perm[s0 + s];
       sx[0].add1(Av0[o]);
       sx[1].add1(Av1[o]);
       sx[2].add1(Av2[o]);
     }
 #pragma unroll
-    for (int m = 8; m > 0; m >>= 1)
+    for (int m = L / 2; m > 0; m >>= 1)
 #pragma unroll
       for (int d = 0; d < 3; ++d) sx[d].combine(sx[d].shfl_xor(m));
     // the shift of the central sums: the mean (FP32 state: the FP32 pair
@@ -3657,7 +3663,7 @@ __global__ void k_moment_sums(StepArgs a, int64_t c0, int64_t c1, double* sums) 
 #pragma unroll
     for (int d = 0; d < K2; ++d) r[d].init();
     if (N >= 2) {
-      for (int s = lane; s < N; s += 16) {
+      for (int s = lane; s < N; s += L) {
         const uint32_t o = a.perm[s0 + s];
         T C0 = Av0[o] - Uh[0], C1 = Av1[o] - Uh[1], C2 = Av2[o] - Uh[2];
         if constexpr (kMixed) {
@@ -3675,7 +3681,7 @@ __global__ void k_moment_sums(StepArgs a, int64_t c0, int64_t c1, double* sums) 
       }
     }
 #pragma unroll
-    for (int m = 8; m > 0; m >>= 1)
+    for (int m = L / 2; m > 0; m >>= 1)
 #pragma unroll
       for (int d = 0; d < K2; ++d) r[d].combine(r[d].shfl_xor(m));
     if (lane == 0 && valid) {
@@ -3827,9 +3833,10 @@ __global__ void k_keys(const T* x0, const T* x1, const T* x2, int64_t M, const u
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t k = kSentinel;
   if (i < M) {
-    const InstParams& P = Ps[part_inst[i]];
+    const InstParams& P = Ps[part_inst ? part_inst[i] : 0u];
     T x[3] = {x0[i], DIM > 1 ? x1[i] : (T)0, DIM > 2 ? x2[i] : (T)0};
-    k = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
+    if constexpr (sizeof(T) == 8) k = (uint32_t)P.cell_off + cell_of_clear<DIM>(P, x);
+    else k = (uint32_t)P.cell_off + cell_of<T, DIM>(P, x);
     key[i] = k;
   }
   warp_count(k, count);  // one atomic per cell per warp (input sorted by cell: few)
@@ -3846,7 +3853,7 @@ __global__ void k_stage_in(const S* pos, const S* vel, int dim, int64_t n, T* p0
   v0[off + j] = (T)vel[j];
   v1[off + j] = (T)vel[n + j];
   v2[off + j] = (T)vel[2 * n + j];
-  part_inst[off + j] = inst;
+  if (part_inst) part_inst[off + j] = inst;
 }
 
 template <class T>

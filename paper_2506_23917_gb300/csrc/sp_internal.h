@@ -231,6 +231,12 @@ void launch_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
                           uint32_t* big_count, uint32_t* ticket, uint32_t* nbatch,
                           double* surf_time, unsigned long long* cyc, cudaStream_t s);
 int64_t scan_partial_size(int64_t n);
+// An upload's particle counts (Mtot = M, Mcur = *kept) and first Delta t (from
+// dt_min, which is reset; *bad = 1 where an instance has neither a cell with
+// two particles nor a fixed step).
+void launch_counts(uint32_t M, const uint32_t* kept, uint32_t* Mtot, uint32_t* Mcur, cudaStream_t s);
+void launch_first_dt(const InstParams* P, int n_inst, double* dt_cur, unsigned long long* dt_min,
+                     unsigned long long* bad, cudaStream_t s);
 
 // Each cell's perm segment in ascending (source) order (sp_noalloc.cu); the
 // small (up to 128 entries) and large cells separately, or both.

@@ -102,7 +102,8 @@ void inject(int dim, const InjectArgs& a, int pass, cudaStream_t s) {
 void moments(const StepArgs& a, int64_t c0, int64_t c1, double* out, cudaStream_t s) {
   const int64_t nc = c1 - c0;
   if (nc <= 0) return;
-  int64_t g = (nc + 15) / 16;  // a half-warp per cell, 16 cells per block, grid-stride
+  constexpr int per = 256 / kMomentLanes<T>;  // cells per block, grid-stride
+  int64_t g = (nc + per - 1) / per;
   if (g > 65535) g = 65535;
   if (out) k_moment_sums<T, A, true><<<(unsigned)g, 256, 0, s>>>(a, c0, c1, a.msum);
   else k_moment_sums<T, A, false><<<(unsigned)g, 256, 0, s>>>(a, c0, c1, a.msum);
