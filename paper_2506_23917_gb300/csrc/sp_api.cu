@@ -7,9 +7,9 @@
 //      DSMC / Shakhov / rescale -> Step 5 sums -> Step 2 free flight of the
 //      next interval, new key and histogram;
 //   2. reservoir injection at inflow faces (count, scan, write);
-//   3. exclusive scan of the histogram -> cell offsets of the new state;
-//   4. bookkeeping (particle count, Delta t of the next step, step index);
-//   5. scatter of source indices into the new cell order (the histogram is
+//   3. exclusive scan of the histogram -> cell offsets of the new state, and
+//      bookkeeping (particle count, Delta t of the next step, step index);
+//   4. scatter of source indices into the new cell order (the histogram is
 //      the cursor and ends at zero, ready for the next step), and in
 //      reproducible runs the source order inside each cell.
 // The sequence is captured once per buffer parity as a CUDA graph and
@@ -574,10 +574,23 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   rec(1);
   if (fork) cudaStreamWaitEvent(c->stream, c->join_ev, 0);
   rec(2);
-  launch_scan(c->count, c->start, c->NC, c->scan_part, c->stream); n += 2;
-  launch_step_finalize(c->dP, c->n_inst, c->dt_cur, c->dt_min, c->step_d, c->Mcur, c->Mtot, c->start,
-                       c->NC, c->goff, c->gcount, c->n_ghost, c->big_count, c->ticket, c->nbatch,
-                       c->surf_time, c->cyc, c->stream); ++n;
+  StepEnd e;
+  e.P = c->dP;
+  e.n_inst = c->n_inst;
+  e.dt_cur = c->dt_cur;
+  e.dt_min = c->dt_min;
+  e.step = c->step_d;
+  e.Mcur = c->Mcur;
+  e.Mtot = c->Mtot;
+  e.goff = c->goff;
+  e.gcount = c->gcount;
+  e.n_ghost = c->n_ghost;
+  e.big_count = c->big_count;
+  e.ticket = c->ticket;
+  e.nbatch = c->nbatch;
+  e.surf_time = c->surf_time;
+  e.cyc = c->cyc;
+  n += launch_scan_end(c->count, c->start, c->NC, c->scan_part, e, c->stream);
   rec(3);
   launch_scatter(c->key[1 - par], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream); ++n;
   if (c->stable) {  // small and large cells side by side

@@ -52,10 +52,47 @@ __global__ void k_scan_reduce(const uint32_t* in, int64_t n, uint32_t* partial) 
   if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
+// End-of-step bookkeeping by one block: particle counts, step index, Delta t
+// of the next step, and the counters of the next step's plan.  kept: the new
+// state's particles (the scan's total).
+__device__ __forceinline__ void step_finalize(const StepEnd& e, uint32_t kept) {
+  const uint32_t st = *e.step;  // index of the step that just ran (read by all first)
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const uint32_t inj = e.n_ghost > 0 ? e.goff[e.n_ghost - 1] + e.gcount[e.n_ghost - 1] : 0u;
+    const uint32_t old = *e.Mcur;
+    *e.Mtot = old + inj;
+    *e.Mcur = kept;
+    *e.step = st + 1u;
+    *e.big_count = 0u;
+    *e.ticket = 0u;
+    for (int k = 0; k < kBatchClasses; ++k) e.nbatch[k] = 0u;
+    // unit of the cost bytes: 1/16 of this step's mean cycles per particle
+    // over all batches (at least 1)
+    const unsigned long long u = e.cyc[1] > 0 ? e.cyc[0] / (16ull * e.cyc[1]) : ~0ull;
+    e.cyc[2] = u > 0 ? u : 1ull;
+    e.cyc[0] = 0ull;
+    e.cyc[1] = 0ull;
+  }
+  for (int i = threadIdx.x; i < e.n_inst; i += blockDim.x) {
+    const unsigned long long inf = 0x7FF0000000000000ull;
+    const InstParams& P = e.P[i];
+    if ((int64_t)st >= (int64_t)P.n_steady) e.surf_time[i] += e.dt_cur[i];
+    if (P.dt_fixed > 0) {
+      e.dt_cur[i] = P.dt_fixed;
+    } else if (e.dt_min[i] != inf) {
+      e.dt_cur[i] = P.cfl * __longlong_as_double((long long)e.dt_min[i]);
+    }
+    e.dt_min[i] = inf;
+  }
+}
+
 // out[j] = sum of in[0..j), out[n] = total.  Each thread owns kScanItems
-// consecutive elements of the block's tile.
+// consecutive elements of the block's tile.  kEnd: the last block, which has
+// the total, also ends the step (a launch of its own took 6 us of every step).
+template <bool kEnd>
 __global__ void k_scan_down(const uint32_t* in, uint32_t* out, int64_t n, const uint32_t* partial,
-                            int64_t nb) {
+                            int64_t nb, StepEnd e) {
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -80,6 +117,9 @@ __global__ void k_scan_down(const uint32_t* in, uint32_t* out, int64_t n, const 
     run += v[i];
   }
   if (blockIdx.x == nb - 1 && threadIdx.x == 0) out[n] = off + tot;
+  if constexpr (kEnd) {
+    if (blockIdx.x == nb - 1) step_finalize(e, off + tot);
+  }
 }
 
 // perm[start[key] + rank] = source index.  The histogram itself is the
@@ -123,41 +163,6 @@ __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* 
   }
 }
 
-__global__ void k_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
-                                unsigned long long* dt_min, uint32_t* step, uint32_t* Mcur,
-                                uint32_t* Mtot, const uint32_t* start_new, int64_t NC,
-                                const uint32_t* goff, const uint32_t* gcount, int64_t n_ghost,
-                                uint32_t* big_count, uint32_t* ticket, uint32_t* nbatch,
-                                double* surf_time, unsigned long long* cyc) {
-  const uint32_t st = *step;  // index of the step that just ran (read by all first)
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const uint32_t inj = n_ghost > 0 ? goff[n_ghost - 1] + gcount[n_ghost - 1] : 0u;
-    const uint32_t old = *Mcur;
-    *Mtot = old + inj;
-    *Mcur = start_new[NC];
-    *step = *step + 1u;
-    *big_count = 0u;
-    *ticket = 0u;
-    for (int k = 0; k < kBatchClasses; ++k) nbatch[k] = 0u;
-    // unit of the cost bytes: 1/16 of this step's mean cycles per particle
-    // over all batches (at least 1)
-    const unsigned long long u = cyc[1] > 0 ? cyc[0] / (16ull * cyc[1]) : ~0ull;
-    cyc[2] = u > 0 ? u : 1ull;
-    cyc[0] = 0ull;
-    cyc[1] = 0ull;
-  }
-  for (int i = threadIdx.x; i < n_inst; i += blockDim.x) {
-    const unsigned long long inf = 0x7FF0000000000000ull;
-    if ((int64_t)st >= (int64_t)P[i].n_steady) surf_time[i] += dt_cur[i];
-    if (P[i].dt_fixed > 0) {
-      dt_cur[i] = P[i].dt_fixed;
-    } else if (dt_min[i] != inf) {
-      dt_cur[i] = P[i].cfl * __longlong_as_double((long long)dt_min[i]);
-    }
-    dt_min[i] = inf;
-  }
-}
 // Work plan of a step: consecutive cells are grouped into batches whose
 // particles fit a warp's staging area (at most 32 cells each); cells above
 // it go to the big-cell list.  One warp per 32-cell chunk.  Each batch is
@@ -349,30 +354,32 @@ void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap
 
 int64_t scan_partial_size(int64_t n) { return (n + kTile - 1) / kTile + 1; }
 
-void launch_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, cudaStream_t s) {
+// (one tile: the down-sweep has no earlier blocks to add)
+static int64_t scan_blocks(const uint32_t* in, int64_t n, uint32_t* partial, cudaStream_t s) {
   const int64_t nb = (n + kTile - 1) / kTile;
-  if (nb == 0) {
+  if (nb > 1) k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, partial);
+  return nb;
+}
+
+void launch_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, cudaStream_t s) {
+  if (n == 0) {
     cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
     return;
   }
-  k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, partial);
-  k_scan_down<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, partial, nb);
+  const int64_t nb = scan_blocks(in, n, partial, s);
+  k_scan_down<false><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, partial, nb, StepEnd());
+}
+
+int launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s) {
+  const int64_t nb = scan_blocks(in, n, partial, s);
+  k_scan_down<true><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, partial, nb, e);
+  return nb > 1 ? 2 : 1;
 }
 
 void launch_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,
                     const uint32_t* Mtot, int64_t cap, cudaStream_t s) {
   const int64_t g = (cap + 256 * kScatterPer - 1) / (256 * kScatterPer);
   k_scatter<<<(unsigned)(g > 0 ? g : 1), 256, 0, s>>>(key, start, count, perm, Mtot, cap);
-}
-
-void launch_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
-                          unsigned long long* dt_min, uint32_t* step, uint32_t* Mcur,
-                          uint32_t* Mtot, const uint32_t* start_new, int64_t NC,
-                          const uint32_t* goff, const uint32_t* gcount, int64_t n_ghost,
-                          uint32_t* big_count, uint32_t* ticket, uint32_t* nbatch,
-                          double* surf_time, unsigned long long* cyc, cudaStream_t s) {
-  k_step_finalize<<<1, 256, 0, s>>>(P, n_inst, dt_cur, dt_min, step, Mcur, Mtot, start_new, NC,
-                                    goff, gcount, n_ghost, big_count, ticket, nbatch, surf_time, cyc);
 }
 
 }  // namespace sp

@@ -224,12 +224,22 @@ void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64
                         double Fn, double R, double* out, cudaStream_t s);
 void launch_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,
                     const uint32_t* Mtot, int64_t cap, cudaStream_t s);
-void launch_step_finalize(const InstParams* P, int n_inst, double* dt_cur,
-                          unsigned long long* dt_min, uint32_t* step, uint32_t* Mcur,
-                          uint32_t* Mtot, const uint32_t* start_new, int64_t NC,
-                          const uint32_t* goff, const uint32_t* gcount, int64_t n_ghost,
-                          uint32_t* big_count, uint32_t* ticket, uint32_t* nbatch,
-                          double* surf_time, unsigned long long* cyc, cudaStream_t s);
+// What the end of a step updates (step_finalize).
+struct StepEnd {
+  const InstParams* P;
+  int n_inst;
+  double* dt_cur;
+  unsigned long long* dt_min;
+  uint32_t *step, *Mcur, *Mtot;
+  const uint32_t *goff, *gcount;
+  int64_t n_ghost;
+  uint32_t *big_count, *ticket, *nbatch;
+  double* surf_time;
+  unsigned long long* cyc;
+};
+// Scan of the new histogram (n > 0 cells) and end of the step; the number of
+// launches.
+int launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s);
 int64_t scan_partial_size(int64_t n);
 // An upload's particle counts (Mtot = M, Mcur = *kept) and first Delta t (from
 // dt_min, which is reset; *bad = 1 where an instance has neither a cell with
