@@ -554,7 +554,14 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
     cudaEventRecord(c->join_ev, c->side);
     n += 4;
   }
-  launch_plan(c->start, c->cost, c->NC, c->sched_cap, small_grid(c) * c->sched_warps, (c->prec != SP_FP64 && c->dim == 2) ? kSplitLanes : 0,
+  // warps among which the plan spreads a small state: with an FP32 state at
+  // most 8 per SM, since every batch costs the FP64 pipe the same per-cell
+  // arithmetic however few its cells (200 k particles, 10 steps: 775 us over
+  // 16 warps per SM, 613 over 8, 604 over 4; the 10-instance ensemble 1516,
+  // 1628, 1923; FP64 mode, whose particles cost more than its cells, all)
+  const int nwarps = small_grid(c) * c->sched_warps;
+  launch_plan(c->start, c->cost, c->NC, c->sched_cap, c->prec != SP_FP64 ? std::min(nwarps, 8 * c->nsm) : nwarps,
+              c->prec != SP_FP64 ? 96 : 32, (c->prec != SP_FP64 && c->dim == 2) ? kSplitLanes : 0,
               c->batches, c->nbatch, c->big_list, c->big_count, c->stream);
   ++n;
   // the big-cell launch (cells disjoint from the batches') is a branch

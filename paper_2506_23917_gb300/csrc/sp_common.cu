@@ -181,12 +181,12 @@ __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* 
 // order changes no result.  A state too small to give every resident warp
 // of the collision launch (nwarps) a full batch is cut into smaller ones,
 // down to one cell each: the launch then lasts as long as one batch, whose
-// time is proportional to its particles (kPlanWaves batches per warp).
-constexpr int kPlanWaves = 1;
-__global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap_max, int nwarps, int split,
-                       uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count) {
-  const int64_t share = ((int64_t)start[NC] + (int64_t)nwarps * kPlanWaves - 1) / ((int64_t)nwarps * kPlanWaves);
-  const int cap = share < 32 ? 32 : share < cap_max ? (int)share : cap_max;
+// time grows with its particles (at least `least` particles, where that many
+// cost no more than fewer).
+__global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap_max, int nwarps, int least,
+                       int split, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count) {
+  const int64_t share = ((int64_t)start[NC] + nwarps - 1) / nwarps, want = share < least ? least : share;
+  const int cap = want < cap_max ? (int)want : cap_max;
   // per block: the batches of each class (shared atomics), then one global
   // atomic per class for the block's place in the class list
   __shared__ uint32_t cnt[kBatchClasses], base[kBatchClasses];
@@ -343,13 +343,13 @@ void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64
   k_mean_fields<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(samp, NC, vol, c0, nc, nsamp, Fn, 3.0 * R, out);
 }
 
-void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int nwarps, int split,
-                 uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
+void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int nwarps, int least,
+                 int split, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
   const int64_t chunks = (NC + 31) / 32;
   int64_t g = (chunks + 7) / 8;
   if (g > 4096) g = 4096;
   if (g < 1) g = 1;
-  k_plan<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, nwarps, split, batches, nbatch, big_list, big_count);
+  k_plan<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, nwarps, least, split, batches, nbatch, big_list, big_count);
 }
 
 int64_t scan_partial_size(int64_t n) { return (n + kTile - 1) / kTile + 1; }
