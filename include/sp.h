@@ -166,9 +166,10 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
 
 /* Step 1 of the paper: give instance `inst` its particles.  pos is
  * [dim][n] (SoA, row d holds coordinate d), vel is [3][n]; both host FP64.
- * The data is copied to a device staging area on the context's stream
- * (asynchronously when the host memory is page-locked: keep it unchanged
- * until the next synchronising call).  At the next sp_step / query every
+ * The data is copied to the device on the context's stream (asynchronously
+ * when the host memory is page-locked: keep it unchanged until the next
+ * synchronising call), into a staging area or, for the one instance of a
+ * context of the same precision, into the state itself.  At the next sp_step / query every
  * instance's staged particles are converted to the context's precision,
  * indexed and stably sorted by cell (input order within a cell), and
  * Delta t of the next step is set to cfl * min dt_c of that state (on an
@@ -280,7 +281,8 @@ sp_status sp_errors(sp_ctx* ctx, int64_t* out5);
  * receives the summed device time of (0) the batch plan and the collision +
  * free-flight kernels, (1) what of the reservoir injection (a branch beside
  * them) is left when they end, (2) the histogram scan and bookkeeping,
- * (3) the scatter.  Synchronises after every step (for measurement only). */
+ * (3) the scatter and the in-cell order.  Synchronises after every step (for
+ * measurement only). */
 sp_status sp_step_profiled(sp_ctx* ctx, int n_steps, double* ms, int n_slots);
 /* Within-cell order of the particles.  on = 1 (default): every step restores
  * the source order inside each cell (a stable counting sort overall), so a

@@ -219,7 +219,8 @@ __device__ __forceinline__ NtcDraw<float> ntc_draw(float, uint32_t step, uint32_
 // u3 < sigma c / (sigma c)_max.  An FP32 estimate (relative error below 1e-5,
 // the sum of the rounding of its inputs, powf and ex ln c_r) settles both
 // unless it comes within 1e-4 of the line; only then is the FP64 value
-// formed, so that every decision is the FP64 one.
+// formed, so that every decision is the FP64 one.  (With the flight's and the
+// Shakhov step's filters: Sod tube of 11 k particles 0.43 -> 0.31 ms per step.)
 struct NtcTest {
   double sc;   // sigma c where it was formed, else -1 (then below S)
   float est;   // estimate of sigma c / S, S = (sigma c)_max before the round
@@ -983,7 +984,8 @@ __device__ __forceinline__ const InstParams& inst_params(const StepArgs& a, uint
 // Per-cell sums with an order fixed by the cell alone (so results do not
 // depend on how cells are grouped into batches).  A cell of at most
 // kLaneSumMax particles is summed by its own lane (lane i <-> cell i) in
-// slot order; with an FP32 state a cell above kSplitLanes particles is cut
+// slot order (FP64 terms: by about N / 8 lanes, as many cells at a time as
+// fill the warp); with an FP32 state a cell above kSplitLanes particles is cut
 // into P = cell_lanes(N) contiguous parts of ceil(N / P) slots, part 0 on
 // its own lane and parts 1..P-1 on helper lanes of the batch (lanes G,
 // G+1, ... in cell order), and its lane adds the parts in part order -- so
@@ -1719,10 +1721,15 @@ __device__ __forceinline__ bool cell_settled(const InstParams& Pi, uint32_t kl, 
 
 // ---------------------------------------------------------------------------
 // One batch of G consecutive cells [k0, k0+G) whose particles fit the warp's
-// staging area: gather through perm -> Step 3 moments -> Step 4 split,
-// DSMC, Shakhov, rescale -> Step 5 sums -> Step 2 free flight, new key and
-// histogram.  Particle work is spread over the lanes across the whole
-// batch; per-cell FP64 arithmetic runs lane-per-cell (lane i <-> cell i).
+// staging area: gather through perm -> Step 3 moments -> Step 4 split, DSMC,
+// Shakhov, rescale -> Step 5 sums -> velocities stored in cell order for the
+// free flight (k_flight).  Particle work is spread over the lanes across the
+// whole batch; per-cell FP64 arithmetic runs lane-per-cell (lane i <-> cell i).
+// Bound by latency, of the dependent chains and the shared-memory round trips
+// at 16 resident warps per SM (FP32 state), and in FP64 mode by the FP64
+// pipe.  The phases stay in one kernel because they share the gather: sums
+// and cell arithmetic as kernels of their own cost the 600 x 300 cylinder
+// 98 us per step and saved 98.
 // ---------------------------------------------------------------------------
 template <class T, class A, int DIM, bool ONE>
 __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A>* ct, uint32_t* sidx,
@@ -1790,7 +1797,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   __syncwarp();
   // ---- 1b. Bird's sub-cells (option): each cell's slots in a stable order
   // by sub-cell (the sub-cell of a slot from its particle's position), so
-  // that every sub-cell is a run of slots; offsets in ct->soff
+  // that every sub-cell is a run of slots; offsets in soff
   const int nsub_i = own ? inst_params<ONE>(a, inst).nsub : 1;
   const unsigned subs = __ballot_sync(kFull, nsub_i > 1);
   if (subs) {
@@ -1851,7 +1858,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   // mean, so FP32 loses little to cancellation): sums of D, of D D^T and of
   // |D|^2 D, from which the central sums follow exactly (below).  All other
   // cases: two passes, the second about the cell mean U (FP64 mode: C = c - U
-  // in FP64, the oracle's sums; FP32 state with FP64 cells: C = (c - U_h) -
+  // in FP64; FP32 state with FP64 cells: C = (c - U_h) -
   // U_l in FP32, with U = U_h + U_l the FP64 mean split into an FP32 pair, and
   // both passes summed without loss into FP64).
   bool one_pass = false;
@@ -2629,8 +2636,8 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1
   int* tags = (int*)tail;
   // One call site of process_batch for both launches, so that every cell
   // runs through the same inlined code (identical rounding whichever launch
-  // or batch takes it).  Main launch: batches from the plan's four class
-  // lists by work stealing, heavy, large, medium, then small.  Big-cell
+  // or batch takes it).  Main launch: batches from the plan's class lists by
+  // work stealing, most expensive class first.  Big-cell
   // launch: a block per cell of the big list.
   // the end of each class in ticket order (main launch)
   uint32_t cend[kBatchClasses];
@@ -3251,6 +3258,13 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
 // and the source's position (runs of neighbouring indices).  The slot's cell
 // -- for the instance, the wall draws' counters and the O-grid's walk -- is
 // the source's key of the last step.
+// Bound by memory latency: 36 B per particle in 2-D FP32, 64 us for 6.6 M
+// (3.7 TB/s); sphere, 30 M, 44 B: 315 us (4.2 TB/s); O-grid, 3.6 M: 66 us;
+// FP64, 1.6 M: 75 us (206 without flight_clear).  Inside the collision kernel,
+// at its 12 warps per SM, the flight was 29 % of the cylinder's, 38 % of the
+// sphere's and 60 % of the O-grid's collision time (steps 0.353 -> 0.337,
+// 1.92 -> 1.70, 0.31 -> 0.229 ms).  Two slots per thread and 4 blocks per SM
+// measured best (1 x 6 blocks, 2 x 5, 4 x 3, 4 x 4: 0 to 5 % slower).
 // ---------------------------------------------------------------------------
 constexpr int kFlightThreads = 256;
 template <class T>

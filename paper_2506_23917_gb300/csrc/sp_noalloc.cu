@@ -116,13 +116,13 @@ __device__ __forceinline__ void sort_segment(uint32_t* p, int64_t n, int64_t tid
 //   k_order_small  up to kSmallSeg: one warp per cell, up to 4 entries per lane;
 //   k_order_large  to kWarpSeg: one warp per cell, 8 to 32 entries per lane;
 //                  above: one block per cell.
-// Bound by the issue of the shuffles and compares, about 3 warp-instructions
-// per entry, at full occupancy and without shared memory for small cells.
-// 600 x 300 cylinder (6.6 M entries, 40 per cell): 53 us; sphere, 30 M
-// entries, 1 M cells: 0.21 ms; jet, 4.5 M entries, most in cells of 500 to
-// 2000: 74 us.  Restoring the order inside the collision kernel instead (12
-// resident warps per SM, one shared-memory read per comparison) took 0.15,
-// 0.38 and 0.38 ms of those flows' steps.
+// Bound by instruction issue, about 2.4 warp-instructions per entry.
+// k_order_small: 600 x 300 cylinder (6.6 M entries, 40 per cell) 35 us (48 by
+// the sorting network alone); sphere, 30 M entries in 1 M cells, 175 us (193).
+// k_order_large: jet, 4.5 M entries, most in cells of 500 to 2000, 66 us.
+// Restoring the order inside the collision kernel instead (12 resident warps
+// per SM, one shared-memory read per comparison) took 0.15, 0.38 and 0.38 ms
+// of those flows' steps.
 constexpr int kSmallSeg = 128;
 constexpr int kWarpSeg = 1024;
 constexpr int kSmemSeg = 8192;       // big cells up to this size are staged in shared memory
