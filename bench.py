@@ -109,7 +109,7 @@ def load_peaks():
 
 
 def collide_profile(src_hash):
-    """Per-particle figures of the collision kernel from the committed ncu
+    """Per-particle figures of the collision and flight kernels from the committed ncu
     summary (DRAM bytes, warp-instructions), if it was taken on the current
     kernel source; else {}."""
     path = os.path.join(ROOT, "profiles", "collide_cylinder_traffic.txt")
@@ -515,7 +515,7 @@ def main():
     step_bytes = (2 * S + 8) * Mp
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": (tpp * Mp) if tpp is not None else None,
-                "kernel": "k_collide (gather + moments + DSMC + Shakhov + rescale + sample + move + key)",
+                "kernel": "k_collide (gather + moments + DSMC + Shakhov + rescale + sample) and k_flight (move + key)",
                 "bytes_per_particle": 2 * S + 4, "peak_source": f"{peak_kind} hbm_gbs",
                 "kernel_ms": collide_ms,
                 "share_of_step": prof[0] / sum(prof),
@@ -523,7 +523,7 @@ def main():
                                       zip(["collide", "inject", "scan", "scatter"], prof)},
                 "step_frac": step_bytes / (step_ms * 1e-3) / 1e9 / peak,
                 "step_bytes_per_particle": 2 * S + 8}
-    # instruction-issue roof of the same kernel: warp-instructions per
+    # instruction-issue roof of the same kernels: warp-instructions per
     # particle (ncu) x particles / kernel time, against SMs x 4 schedulers x
     # the SM clock under load (one warp-instruction per scheduler per cycle)
     ipp = prof_pp.get("inst_per_particle")
