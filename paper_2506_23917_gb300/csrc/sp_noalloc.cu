@@ -82,40 +82,12 @@ __global__ void __launch_bounds__(kStaticThreads) k_static_scatter(const uint32_
   }
 }
 
-// In-place sorting network whose comparators all point the same way (each
-// stage first compares slot t with its mirror t ^ (k-1) inside the current
-// block of k slots, then runs the half-cleaners): it sorts a segment of any
-// length n without padding, the slots past the end acting as +infinity.
-// Thread `tid` of `nthr` cooperating threads takes slots tid, tid + nthr, ...;
-// `sync` separates the stages.  All sizes are 64-bit, so segments up to the
-// entry point's limit of 2^30 entries cannot overflow the loop bounds.
-template <class Sync>
-__device__ __forceinline__ void sort_segment(uint32_t* p, int64_t n, int64_t tid, int64_t nthr, Sync sync) {
-  int64_t n2 = 1;
-  while (n2 < n) n2 <<= 1;
-  for (int64_t k = 2; k <= n2; k <<= 1) {
-    for (int64_t j = k >> 1; j > 0; j >>= 1) {
-      for (int64_t t = tid; t < n; t += nthr) {
-        const int64_t q = (j == (k >> 1)) ? (t ^ (k - 1)) : (t ^ j);
-        if (q > t && q < n) {
-          const uint32_t a = p[t], b = p[q];
-          if (a > b) {
-            p[t] = b;
-            p[q] = a;
-          }
-        }
-      }
-      sync();
-    }
-  }
-}
-
 // Stable order of the cells' entries.  The scatter's atomics leave each
 // cell's source indices in arbitrary order; two kernels over disjoint cell
 // sizes put them in ascending order:
 //   k_order_small  up to kSmallSeg: one warp per cell, up to 4 entries per lane;
 //   k_order_large  to kWarpSeg: one warp per cell, 8 to 32 entries per lane;
-//                  above: one block per cell.
+//                  above: one block per cell (order_chunk, order_chunks).
 // Bound by instruction issue, about 2.4 warp-instructions per entry.
 // k_order_small: 600 x 300 cylinder (6.6 M entries, 40 per cell) 35 us (48 by
 // the sorting network alone); sphere, 30 M entries in 1 M cells, 175 us (193).
@@ -125,7 +97,7 @@ __device__ __forceinline__ void sort_segment(uint32_t* p, int64_t n, int64_t tid
 // of those flows' steps.
 constexpr int kSmallSeg = 128;
 constexpr int kWarpSeg = 1024;
-constexpr int kSmemSeg = 8192;       // big cells up to this size are staged in shared memory
+constexpr int kSmemSeg = 8192;       // entries a block stages in shared memory
 constexpr int kOrderWarps = 8;
 constexpr int kOrderThreads = 32 * kOrderWarps;
 constexpr int kOrderSmem = kSmemSeg + kSmemSeg / 32;  // words: a pad word every 32
@@ -137,9 +109,11 @@ __device__ __forceinline__ void lo_hi(uint32_t& a, uint32_t& b) {
 }
 
 // Ascending sort of 32 R entries held by a warp, entry lane R + i in x[i]
-// (any assignment of the input to lanes will do): the network of
-// sort_segment, with the stages inside a lane on registers and the others
-// by shuffles.
+// (any assignment of the input to lanes will do), by a network whose
+// comparators all point the same way: for blocks of k = 2, 4, ... slots, each
+// slot t is first compared with its mirror t ^ (k - 1) inside its block, then
+// with t ^ j for j = k/4, k/8, ... 1.  The stages inside a lane run on
+// registers, the others by shuffles.
 template <int R>
 __device__ __forceinline__ void warp_sort(uint32_t (&x)[R], int lane) {
 #pragma unroll
@@ -353,12 +327,76 @@ __device__ __forceinline__ void order_block(uint32_t* g, int n, uint32_t* seg) {
   __syncthreads();
 }
 
-__device__ __forceinline__ void order_big_cell(uint32_t* g, int64_t n, uint32_t* seg) {
+__device__ __forceinline__ void order_chunk(uint32_t* g, int n, uint32_t* seg) {
   static_assert(kSmemSeg == kOrderWarps * 1024 && kWarpSeg < kOrderWarps * 256, "runs of one warp each");
-  if (n <= kOrderWarps * 256) order_block<8>(g, (int)n, seg);
-  else if (n <= kOrderWarps * 512) order_block<16>(g, (int)n, seg);
-  else if (n <= kSmemSeg) order_block<32>(g, (int)n, seg);
-  else sort_segment(g, n, threadIdx.x, kOrderThreads, [] { __syncthreads(); });
+  if (n <= kOrderWarps * 256) order_block<8>(g, n, seg);
+  else if (n <= kOrderWarps * 512) order_block<16>(g, n, seg);
+  else order_block<32>(g, n, seg);
+}
+
+// Puts slots t < q of each pair p < pairs (tq(p, &t, &q)) in order, except
+// where q >= n; a thread's four pairs are loaded together.
+template <class TQ, class At>
+__device__ __forceinline__ void compare_pairs(uint32_t pairs, uint32_t n, TQ tq, At at) {
+  constexpr int U = 4;
+  for (uint32_t p0 = threadIdx.x; p0 < pairs; p0 += U * kOrderThreads) {
+    uint32_t t[U], q[U], x[U], y[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t p = p0 + u * kOrderThreads;
+      tq(p, &t[u], &q[u]);
+      const bool ok = p < pairs && q[u] < n;
+      x[u] = ok ? at(t[u]) : 0u;
+      y[u] = ok ? at(q[u]) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (x[u] > y[u]) {
+        at(t[u]) = y[u];
+        at(q[u]) = x[u];
+      }
+  }
+  __syncthreads();
+}
+
+// A cell above kSmemSeg entries (of any length: slots past n act as the
+// largest value): chunks of kSmemSeg are put in order one by one, then merged
+// by the remaining stages of warp_sort's network, those that compare across
+// chunks in global memory (one to log2(n / kSmemSeg) per doubling) and the 13
+// inside a chunk in shared memory.  Bound by the one block's latency.  One
+// cell of 98,304 entries 1.2 ms, of 2^20 18 ms (the whole network in global
+// memory, 153 and 210 passes: 10.7 and 151 ms; with 512 threads 7.3 and 97);
+// 400 cells of 40,000 entries at random 5.6 ms (10.3; 8.0).
+__device__ __forceinline__ void order_chunks(uint32_t* g, uint32_t n, uint32_t* seg) {
+  for (uint32_t c = 0; c < n; c += kSmemSeg) order_chunk(g + c, (int)(n - c < kSmemSeg ? n - c : kSmemSeg), seg);
+  for (uint64_t k = 2 * kSmemSeg; k < 2 * (uint64_t)n; k <<= 1) {
+    for (uint32_t j = (uint32_t)(k >> 1); j >= kSmemSeg; j >>= 1) {
+      const uint32_t flip = 2 * (uint64_t)j == k ? (uint32_t)(k - 1) : j;
+      compare_pairs((uint32_t)(((uint64_t)n + 2 * (uint64_t)j - 1) / (2 * (uint64_t)j) * j), n,
+                    [&](uint32_t p, uint32_t* t, uint32_t* q) {
+                      *t = (p & (0u - j)) << 1 | (p & (j - 1));
+                      *q = *t ^ flip;
+                    },
+                    [&](uint32_t e) -> uint32_t& { return g[e]; });
+    }
+    const auto at = [&](uint32_t e) -> uint32_t& { return seg[e + (e >> 5)]; };
+    for (uint32_t c = 0; c < n; c += kSmemSeg) {
+      const uint32_t m = n - c < kSmemSeg ? n - c : kSmemSeg;
+#pragma unroll 4
+      for (uint32_t t = threadIdx.x; t < m; t += kOrderThreads) at(t) = g[c + t];
+      __syncthreads();
+      for (uint32_t j = kSmemSeg >> 1; j > 0; j >>= 1)
+        compare_pairs(kSmemSeg / 2, m,
+                      [&](uint32_t p, uint32_t* t, uint32_t* q) {
+                        *t = (p & (0u - j)) << 1 | (p & (j - 1));
+                        *q = *t | j;
+                      },
+                      at);
+#pragma unroll 4
+      for (uint32_t t = threadIdx.x; t < m; t += kOrderThreads) g[c + t] = at(t);
+      __syncthreads();
+    }
+  }
 }
 
 // Cells up to kSmallSeg entries: a warp takes kOrderCells consecutive cells
@@ -435,7 +473,9 @@ __global__ void __launch_bounds__(kOrderThreads, 4) k_order_large(const uint32_t
       const int nl = nlist;
       for (int q = 0; q < nl; ++q) {
         const int64_t k = (int64_t)list[q];
-        order_big_cell(perm + start[k], (int64_t)(start[k + 1] - start[k]), sh);
+        const uint32_t n = start[k + 1] - start[k];
+        if (n <= (uint32_t)kSmemSeg) order_chunk(perm + start[k], (int)n, sh);
+        else order_chunks(perm + start[k], n, sh);
       }
       __syncthreads();
     }
