@@ -723,7 +723,7 @@ sp_status upload(sp_ctx* c) {
   }
   // Delta t from the moments of this state
   const StepArgs a = make_step_args(c, c->cur);
-  c->K->moments(a, 0, c->NC, nullptr, c->stream);
+  c->K->moments(a, 0, c->NC, nullptr, c->nsm, c->stream);
   volatile unsigned long long* bad = c->herr + kNumErr;
   *bad = 0;
   launch_first_dt(c->dP, c->n_inst, c->dt_cur, c->dt_min, c->herr_dev + kNumErr, c->stream);
@@ -1244,7 +1244,7 @@ sp_status sp_moments(sp_ctx* c, int inst, int kind, double* out, int n_fields) {
     // (reproducible runs: every step leaves the cells in source order, so
     // each cell is summed in that order)
     const StepArgs a = make_step_args(c, c->cur);
-    c->K->moments(a, P.cell_off, P.cell_off + nc, d, c->stream);
+    c->K->moments(a, P.cell_off, P.cell_off + nc, d, c->nsm, c->stream);
   } else {
     const int64_t nsamp = std::max<int64_t>(0, c->step_host - (int64_t)P.n_steady);
     launch_mean_fields(c->samp, c->NC, c->vol, P.cell_off, nc, (double)nsamp, P.Fn, P.R, d, c->stream);

@@ -3601,10 +3601,11 @@ __global__ void k_keys_mesh(const T* x0, const T* x1, int64_t M, const uint32_t*
 // Observability / initialisation kernels
 // ---------------------------------------------------------------------------
 // Moments of the current state for cells [c0, c1), in the cells' current
-// slot order, in two kernels.  k_moment_sums: kMomentLanes lanes per
-// cell; lanes stride over the cell's slots, a butterfly combines them, and
-// the first lane writes the cell's sums to sums[7][nc]: sum c (3), then
-// sum |C|^2 and, when the fields are wanted (kQ), sum |C|^2 C (3) about
+// slot order, in two kernels.  k_moment_sums: kMomentLanes lanes per cell (a
+// warp per dense cell of an FP64 state); lanes stride over the cell's slots, a
+// butterfly combines them, and the first lane writes the cell's sums to
+// sums[7][nc]: sum c (3), then sum |C|^2 and, when the fields are wanted (kQ),
+// sum |C|^2 C (3) about
 // the mean.  The sums use the
 // collision kernel's accumulators (FP64 values in FP64 mode, FP32 terms
 // carried without loss in FP32 mode, plain FP32 in the all-FP32 mode).
@@ -3618,99 +3619,131 @@ __global__ void k_keys_mesh(const T* x0, const T* x1, int64_t M, const uint32_t*
 // minimum dt_c into dt_min (a warp minimum, then one atomic per warp).
 // Lanes per cell: 16 with an FP32 state; 4 with an FP64 state, where the
 // butterfly's additions hold the FP64 pipe as long as the terms' (2 M
-// particles, 30 per cell: 221 -> 118 us with the heat flux).
+// particles, 30 per cell: 221 -> 118 us with the heat flux), and 32 for its
+// cells above kMomentDense particles, whose time is the gathers of one lane.
+// Reads of an FP64 state with 16, 4 and these lanes: one cell of 200,000 21.1,
+// 35.7 and 4.6 ms; 267 cells of 1500 240, 615 and 123 us; 2000 of 200 120, 134
+// and 83 us; 5000 of 80 123, 87 and 88 us.  Four rounds of gathers are in
+// flight (one: 20 to 60 % slower on dense cells; eight: 10 % slower on others).
 template <class T>
 constexpr int kMomentLanes = sizeof(T) == 8 ? 4 : 16;
+constexpr int kMomentDense = 128;
 
-template <class T, class A, bool kQ>
-__global__ void k_moment_sums(StepArgs a, int64_t c0, int64_t c1, double* sums) {
+// One cell of N particles from slot s0 on, by L neighbouring lanes of a warp
+// (`lane` of L); the whole warp calls it (N = 0 where a group has no cell).
+// store: write the sums to sums[..][i].
+template <class T, class A, bool kQ, int L>
+__device__ __forceinline__ void moment_cell(const StepArgs& a, uint32_t s0, int N, int lane, bool store, int64_t i,
+                                            int64_t nc, double* sums) {
   using Acc = CellAcc<T, A>;
   constexpr bool kMixed = mixed_prec<T, A>();
   constexpr bool kPair = sizeof(T) == 4;
-  constexpr int L = kMomentLanes<T>, W = 32 / L;  // lanes per cell, cells per warp
-  const int lane = threadIdx.x & (L - 1);
-  const int64_t nh = (int64_t)gridDim.x * (blockDim.x / L);
-  const int64_t nc = c1 - c0;
   const T* Av0 = (const T*)a.Avel[0];
   const T* Av1 = (const T*)a.Avel[1];
   const T* Av2 = (const T*)a.Avel[2];
-  // the same trip count for all cells of a warp (the shuffles need all lanes)
-  const int64_t h0 = (int64_t)blockIdx.x * (blockDim.x / L) + threadIdx.x / L;
-  for (int64_t kb = c0 + (h0 & ~(int64_t)(W - 1)); kb < c1; kb += nh) {
-    const int64_t k = kb + (h0 & (W - 1));
-    const bool valid = k < c1;
-    const uint32_t s0 = valid ? a.start[k] : 0u;
-    const int N = valid ? (int)(a.start[k + 1] - s0) : 0;
-    Acc sx[3];
+  Acc sx[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) sx[d].init();
+  for (int d = 0; d < 3; ++d) sx[d].init();
+#pragma unroll 4
+  for (int s = lane; s < N; s += L) {
+    const uint32_t o = a.perm[s0 + s];
+    sx[0].add1(Av0[o]);
+    sx[1].add1(Av1[o]);
+    sx[2].add1(Av2[o]);
+  }
+#pragma unroll
+  for (int m = L / 2; m > 0; m >>= 1)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) sx[d].combine(sx[d].shfl_xor(m));
+  // the shift of the central sums: the mean (FP32 state: the FP32 pair
+  // U_h + U_l of the exact sum, formed without FP64 work)
+  T Uh[3] = {0, 0, 0}, Ul[3] = {0, 0, 0};
+  if (N > 0) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if constexpr (kMixed) {
+        const float fN = (float)N, rN = 1.0f / fN;
+        Uh[d] = sx[d].s * rN;
+        Ul[d] = (fmaf(-Uh[d], fN, sx[d].s) + sx[d].e) * rN;
+      } else if constexpr (kPair) {
+        Uh[d] = sx[d].get() * (1.0f / (float)N);
+      } else {
+        Uh[d] = (T)((double)sx[d].get() / N);
+      }
+    }
+  }
+  // sum |C|^2, and with kQ sum |C|^2 C (the heat flux; not needed for dt_c)
+  constexpr int K2 = kQ ? 4 : 1;
+  Acc r[K2];
+#pragma unroll
+  for (int d = 0; d < K2; ++d) r[d].init();
+  if (N >= 2) {
+#pragma unroll 4
     for (int s = lane; s < N; s += L) {
       const uint32_t o = a.perm[s0 + s];
-      sx[0].add1(Av0[o]);
-      sx[1].add1(Av1[o]);
-      sx[2].add1(Av2[o]);
-    }
-#pragma unroll
-    for (int m = L / 2; m > 0; m >>= 1)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) sx[d].combine(sx[d].shfl_xor(m));
-    // the shift of the central sums: the mean (FP32 state: the FP32 pair
-    // U_h + U_l of the exact sum, formed without FP64 work)
-    T Uh[3] = {0, 0, 0}, Ul[3] = {0, 0, 0};
-    if (N > 0) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        if constexpr (kMixed) {
-          const float fN = (float)N, rN = 1.0f / fN;
-          Uh[d] = sx[d].s * rN;
-          Ul[d] = (fmaf(-Uh[d], fN, sx[d].s) + sx[d].e) * rN;
-        } else if constexpr (kPair) {
-          Uh[d] = sx[d].get() * (1.0f / (float)N);
-        } else {
-          Uh[d] = (T)((double)sx[d].get() / N);
-        }
+      T C0 = Av0[o] - Uh[0], C1 = Av1[o] - Uh[1], C2 = Av2[o] - Uh[2];
+      if constexpr (kMixed) {
+        C0 -= Ul[0];
+        C1 -= Ul[1];
+        C2 -= Ul[2];
+      }
+      const T c2 = C0 * C0 + C1 * C1 + C2 * C2;
+      r[0].add1(c2);
+      if constexpr (kQ) {
+        r[1].add1(c2 * C0);
+        r[2].add1(c2 * C1);
+        r[3].add1(c2 * C2);
       }
     }
-    // sum |C|^2, and with kQ sum |C|^2 C (the heat flux; not needed for dt_c)
-    constexpr int K2 = kQ ? 4 : 1;
-    Acc r[K2];
+  }
 #pragma unroll
-    for (int d = 0; d < K2; ++d) r[d].init();
-    if (N >= 2) {
-      for (int s = lane; s < N; s += L) {
-        const uint32_t o = a.perm[s0 + s];
-        T C0 = Av0[o] - Uh[0], C1 = Av1[o] - Uh[1], C2 = Av2[o] - Uh[2];
-        if constexpr (kMixed) {
-          C0 -= Ul[0];
-          C1 -= Ul[1];
-          C2 -= Ul[2];
-        }
-        const T c2 = C0 * C0 + C1 * C1 + C2 * C2;
-        r[0].add1(c2);
-        if constexpr (kQ) {
-          r[1].add1(c2 * C0);
-          r[2].add1(c2 * C1);
-          r[3].add1(c2 * C2);
-        }
-      }
+  for (int m = L / 2; m > 0; m >>= 1)
+#pragma unroll
+    for (int d = 0; d < K2; ++d) r[d].combine(r[d].shfl_xor(m));
+  if (lane == 0 && store) {
+    if constexpr (kPair) {
+      float2* sp2 = (float2*)sums;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) sp2[d * nc + i] = acc_pair(sx[d]);
+#pragma unroll
+      for (int d = 0; d < K2; ++d) sp2[(3 + d) * nc + i] = acc_pair(r[d]);
+    } else {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) sums[d * nc + i] = (double)sx[d].get();
+#pragma unroll
+      for (int d = 0; d < K2; ++d) sums[(3 + d) * nc + i] = (double)r[d].get();
     }
-#pragma unroll
-    for (int m = L / 2; m > 0; m >>= 1)
-#pragma unroll
-      for (int d = 0; d < K2; ++d) r[d].combine(r[d].shfl_xor(m));
-    if (lane == 0 && valid) {
-      const int64_t i = k - c0;
-      if constexpr (kPair) {
-        float2* sp2 = (float2*)sums;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) sp2[d * nc + i] = acc_pair(sx[d]);
-#pragma unroll
-        for (int d = 0; d < K2; ++d) sp2[(3 + d) * nc + i] = acc_pair(r[d]);
-      } else {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) sums[d * nc + i] = (double)sx[d].get();
-#pragma unroll
-        for (int d = 0; d < K2; ++d) sums[(3 + d) * nc + i] = (double)r[d].get();
+  }
+}
+
+// A warp takes G cells at a time: one per group of L lanes (W), or fewer
+// where dense cells (FP64 state: above kMomentDense on average) are too few
+// to give every warp of the launch W of them.  Which cells share a warp does
+// not change how a cell is summed.
+template <class T, class A, bool kQ>
+__global__ void k_moment_sums(StepArgs a, int64_t c0, int64_t c1, double* sums) {
+  constexpr int L = kMomentLanes<T>, W = 32 / L;
+  constexpr bool kDense = sizeof(T) == 8;
+  const int64_t nc = c1 - c0, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  int G = W;
+  if (kDense && (int64_t)(a.start[c1] - a.start[c0]) > kMomentDense * nc) {
+    const int64_t g = (nc + nw - 1) / nw;
+    if (g < W) G = (int)g;
+  }
+  const int wl = threadIdx.x & 31, lane = wl & (L - 1), grp = wl / L;
+  // (the same trip count for all lanes of a warp: the shuffles need them)
+  for (int64_t kb = c0 + ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * G; kb < c1; kb += nw * G) {
+    const int64_t k = kb + grp;
+    const bool valid = grp < G && k < c1;
+    const uint32_t s0 = valid ? a.start[k] : 0u;
+    const int N = valid ? (int)(a.start[k + 1] - s0) : 0;
+    const bool dense = kDense && N > kMomentDense;
+    moment_cell<T, A, kQ, L>(a, s0, dense ? 0 : N, lane, valid && !dense, k - c0, nc, sums);
+    if constexpr (kDense) {
+      for (unsigned todo = __ballot_sync(kFull, dense && lane == 0); todo; todo &= todo - 1) {
+        const int src = __ffs((int)todo) - 1;
+        moment_cell<T, A, kQ, 32>(a, __shfl_sync(kFull, s0, src), __shfl_sync(kFull, N, src), wl, true,
+                                  kb + src / L - c0, nc, sums);
       }
     }
   }

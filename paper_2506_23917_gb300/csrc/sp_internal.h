@@ -199,7 +199,7 @@ struct KernelSet {
   int (*collide_blocks_per_sm)(int dim, int warps, int cap, bool one, bool subcells);
   cudaError_t (*configure)();
   void (*inject)(int dim, const InjectArgs& a, int pass, cudaStream_t s);
-  void (*moments)(const StepArgs& a, int64_t c0, int64_t c1, double* out, cudaStream_t s);
+  void (*moments)(const StepArgs& a, int64_t c0, int64_t c1, double* out, int nsm, cudaStream_t s);
   void (*keys)(int dim, const void* const pos[3], int64_t M, const uint32_t* part_inst, const InstParams* P,
                uint32_t* key, uint32_t* count, cudaStream_t s);
   void (*keys_mesh)(const void* const pos[3], int64_t M, const uint32_t* part_inst, const InstParams* P,

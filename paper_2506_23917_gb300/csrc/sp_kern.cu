@@ -3,6 +3,8 @@
 //   SP_KT  particle state and per-particle arithmetic (float or double),
 //   SP_KA  per-cell sums and per-cell arithmetic (float or double),
 //   SP_TAG suffix of the exported kernel table (f64, f32, f32c).
+#include <algorithm>
+
 #include "sp_device.cuh"
 
 #if !defined(SP_KT) || !defined(SP_KA) || !defined(SP_TAG)
@@ -99,11 +101,13 @@ void inject(int dim, const InjectArgs& a, int pass, cudaStream_t s) {
   else inject_dim<3>(a, pass, s);
 }
 
-void moments(const StepArgs& a, int64_t c0, int64_t c1, double* out, cudaStream_t s) {
+void moments(const StepArgs& a, int64_t c0, int64_t c1, double* out, int nsm, cudaStream_t s) {
   const int64_t nc = c1 - c0;
   if (nc <= 0) return;
   constexpr int per = 256 / kMomentLanes<T>;  // cells per block, grid-stride
   int64_t g = (nc + per - 1) / per;
+  if (sizeof(T) == 8)  // a warp per cell while four blocks per SM are not filled (dense cells)
+    g = std::max(g, std::min<int64_t>((nc + 7) / 8, 4 * nsm));
   if (g > 65535) g = 65535;
   if (out) k_moment_sums<T, A, true><<<(unsigned)g, 256, 0, s>>>(a, c0, c1, a.msum);
   else k_moment_sums<T, A, false><<<(unsigned)g, 256, 0, s>>>(a, c0, c1, a.msum);
