@@ -95,7 +95,6 @@ struct sp_ctx {
   std::vector<double*> dstage;    // per instance: FP64 [dim][n] then [3][n], device
   std::vector<int64_t> stage_n, stage_cap;
   std::vector<int> stage_f32;     // per instance: the staged data is FP32
-  uint32_t* part_inst = nullptr;  // [cap] instance of each uploaded particle
   std::vector<uint32_t> prev_start;  // [NC+1] of the state before the last step (record mode)
   // body-fitted O-grid instances (all instances share the mesh kind)
   int mesh = 0;
@@ -682,6 +681,9 @@ sp_status upload(sp_ctx* c) {
   if (M > c->cap) return SP_ERR_CAPACITY;
   const int dim = c->dim;
   cudaStream_t ix = c->stream;  // where the cells are indexed
+  // the instance of each particle: in the other buffer's keys, which the next
+  // step overwrites (an array of its own cost 4 bytes per slot)
+  uint32_t* part_inst = c->n_inst > 1 ? c->key[1 - c->cur] : nullptr;
   if (c->direct) {
     // the positions were copied first: index the cells while the velocities
     // are on their way
@@ -695,9 +697,9 @@ sp_status upload(sp_ctx* c) {
         const double* sp = c->dstage[i];
         const float* sf = (const float*)c->dstage[i];
         if (c->stage_f32[i])
-          c->K->stage_in32(dim, sf, sf + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst, (uint32_t)i, ix);
+          c->K->stage_in32(dim, sf, sf + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, part_inst, (uint32_t)i, ix);
         else
-          c->K->stage_in(dim, sp, sp + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, c->part_inst, (uint32_t)i, ix);
+          c->K->stage_in(dim, sp, sp + dim * n, n, c->pos[c->cur], c->vel[c->cur], off, part_inst, (uint32_t)i, ix);
       }
       off += n;
     }
@@ -705,9 +707,9 @@ sp_status upload(sp_ctx* c) {
   CK(cudaMemsetAsync(c->count, 0, sizeof(uint32_t) * c->NC, ix));
   const void* P3[3] = {c->pos[c->cur][0], c->pos[c->cur][1], c->pos[c->cur][2]};
   if (c->mesh)
-    c->K->keys_mesh(P3, M, c->part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key[c->cur], c->count, ix);
+    c->K->keys_mesh(P3, M, part_inst, c->dP, c->mface, c->mnode, c->mrad, c->key[c->cur], c->count, ix);
   else
-    c->K->keys(dim, P3, M, c->part_inst, c->dP, c->key[c->cur], c->count, ix);
+    c->K->keys(dim, P3, M, part_inst, c->dP, c->key[c->cur], c->count, ix);
   launch_scan(c->count, c->start, c->NC, c->scan_part, ix);
   // the state holds the located particles only: an O-grid drops those
   // outside the mesh (sentinel keys), so its size is start[NC], not M
@@ -867,7 +869,6 @@ sp_status sp_init(const sp_config* cfgs, int n_instances, int precision, int64_t
         CK(dalloc(&c->vel[b][d], cap * c->tsize));
       }
     for (int b = 0; b < 2; ++b) CK(dalloc(&c->key[b], 4 * cap));
-    if (n_instances > 1) CK(dalloc(&c->part_inst, 4 * cap));
     CK(dalloc(&c->perm, 4 * cap));
     CK(dalloc(&c->count, 4 * NC));
     CK(dalloc(&c->start, 4 * (NC + 1)));
@@ -1470,7 +1471,7 @@ sp_status sp_free(sp_ctx* c) {
       cudaFree(c->vel[b][d]);
     }
   for (double* p : c->dstage) cudaFree(p);
-  void* ptrs[] = {c->Lc, c->iLc, c->mrad, c->mface, c->mnode, c->ivol, c->rcp, c->cons, c->mom, c->msum, c->cost, c->cyc, c->surf, c->surf_time, c->batches, c->nbatch, c->ticket, c->part_inst, c->key[0], c->key[1], c->perm, c->count, c->start, c->cell_inst, c->scan_part, c->big_list,
+  void* ptrs[] = {c->Lc, c->iLc, c->mrad, c->mface, c->mnode, c->ivol, c->rcp, c->cons, c->mom, c->msum, c->cost, c->cyc, c->surf, c->surf_time, c->batches, c->nbatch, c->ticket, c->key[0], c->key[1], c->perm, c->count, c->start, c->cell_inst, c->scan_part, c->big_list,
                   c->big_count, c->vol, c->smax, c->rem, c->samp, c->rec, c->resamp, c->dP, c->dt_cur, c->dt_min,
                   c->step_d, c->Mcur, c->Mtot, c->err, c->ghosts, c->gcount, c->goff, c->gscan_part};
   for (void* p : ptrs) cudaFree(p);
