@@ -530,8 +530,7 @@ bool apply_schedule(sp_ctx* c, int cap, int warps) {
 // ev[0..4] bracket the four kernel groups (the plan and collision
 // launches; what is left of the injection branch when they end; the scan
 // and bookkeeping; the scatter), so that the host can time them.
-int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
-  int n = 0;
+void enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   const StepArgs a = make_step_args(c, par);
   const auto rec = [&](int k) {
     if (ev) cudaEventRecordWithFlags(ev[k], c->stream, cudaEventRecordExternal);
@@ -551,7 +550,6 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
     launch_scan(c->gcount, c->goff, c->n_ghost, c->gscan_part, c->side);
     c->K->inject(c->dim, ia, 1, c->side);
     cudaEventRecord(c->join_ev, c->side);
-    n += 4;
   }
   // warps among which the plan spreads a small state: with an FP32 state at
   // most 8 per SM, since every batch costs the FP64 pipe the same per-cell
@@ -562,21 +560,20 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   launch_plan(c->start, c->cost, c->NC, c->sched_cap, c->prec != SP_FP64 ? std::min(nwarps, 8 * c->nsm) : nwarps,
               c->prec != SP_FP64 ? 96 : 32, (c->prec != SP_FP64 && c->dim == 2) ? kSplitLanes : 0,
               c->batches, c->nbatch, c->big_list, c->big_count, c->stream);
-  ++n;
   // the big-cell launch (cells disjoint from the batches') is a branch
   // beside the main launch: its blocks start as SMs free up at the end of
   // the main launch instead of after all of it
   cudaEventRecord(c->fork2_ev, c->stream);
   cudaStreamWaitEvent(c->side2, c->fork2_ev, 0);
   cudaStreamWaitEvent(c->side3, c->fork2_ev, 0);
-  launch_collide_p(c, a, true, kBigGridPerSm * c->nsm, c->side2); ++n;
+  launch_collide_p(c, a, true, kBigGridPerSm * c->nsm, c->side2);
   cudaEventRecord(c->join2_ev, c->side2);
-  c->K->collide_huge(c->dim, a, kBigGridPerSm * c->nsm, c->side3); ++n;
+  c->K->collide_huge(c->dim, a, kBigGridPerSm * c->nsm, c->side3);
   cudaEventRecord(c->join3_ev, c->side3);
-  launch_collide_p(c, a, false, small_grid(c), c->stream); ++n;
+  launch_collide_p(c, a, false, small_grid(c), c->stream);
   cudaStreamWaitEvent(c->stream, c->join2_ev, 0);
   cudaStreamWaitEvent(c->stream, c->join3_ev, 0);
-  c->K->flight(c->dim, a, c->nsm, c->stream); ++n;
+  c->K->flight(c->dim, a, c->nsm, c->stream);
   rec(1);
   if (fork) cudaStreamWaitEvent(c->stream, c->join_ev, 0);
   rec(2);
@@ -596,19 +593,18 @@ int enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   e.nbatch = c->nbatch;
   e.surf_time = c->surf_time;
   e.cyc = c->cyc;
-  n += launch_scan_end(c->count, c->start, c->NC, c->scan_part, e, c->stream);
+  launch_scan_end(c->count, c->start, c->NC, c->scan_part, e, c->stream);
   rec(3);
-  launch_scatter(c->key[1 - par], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream); ++n;
+  launch_scatter(c->key[1 - par], c->start, c->count, c->perm, c->Mtot, c->cap, c->stream);
   if (c->stable) {  // small and large cells side by side
     cudaEventRecord(c->fork3_ev, c->stream);
     cudaStreamWaitEvent(c->side2, c->fork3_ev, 0);
-    launch_order_large(c->start, c->NC, c->perm, c->side2); ++n;
+    launch_order_large(c->start, c->NC, c->perm, c->side2);
     cudaEventRecord(c->join2_ev, c->side2);
-    launch_order_small(c->start, c->NC, c->perm, c->stream); ++n;
+    launch_order_small(c->start, c->NC, c->perm, c->stream);
     cudaStreamWaitEvent(c->stream, c->join2_ev, 0);
   }
   rec(4);
-  return n;
 }
 
 void destroy_graphs(sp_ctx* c) {
@@ -634,6 +630,21 @@ sp_status make_streams(sp_ctx* c) {
   return SP_OK;
 }
 
+// The kernel nodes of a captured step: its launches.
+cudaError_t count_kernels(cudaGraph_t g, int* kernels) {
+  size_t n = 0;
+  cudaError_t e = cudaGraphGetNodes(g, nullptr, &n);
+  std::vector<cudaGraphNode_t> nodes(n);
+  if (e == cudaSuccess) e = cudaGraphGetNodes(g, nodes.data(), &n);
+  *kernels = 0;
+  for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+    cudaGraphNodeType t;
+    e = cudaGraphNodeGetType(nodes[i], &t);
+    *kernels += e == cudaSuccess && t == cudaGraphNodeTypeKernel;
+  }
+  return e;
+}
+
 // Capture the step graphs of both buffer parities; prof: the copies with
 // timing events at the kernel groups' boundaries (built when first wanted).
 sp_status build_graphs(sp_ctx* c, bool prof = false) {
@@ -649,14 +660,14 @@ sp_status build_graphs(sp_ctx* c, bool prof = false) {
     cudaGraph_t g;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      const int n = enqueue_step(c, par, prof ? c->pev : nullptr);
-      c->launches = n;
+      enqueue_step(c, par, prof ? c->pev : nullptr);
       e = cudaStreamEndCapture(cs, &g);
     }
     c->stream = saved;
     cudaStreamDestroy(cs);
     CK(e);
-    e = cudaGraphInstantiate(&out[par], g, 0);
+    e = count_kernels(g, &c->launches);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&out[par], g, 0);
     cudaGraphDestroy(g);
     CK(e);
   }

@@ -370,10 +370,9 @@ void launch_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial
   k_scan_down<false><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, partial, nb, StepEnd());
 }
 
-int launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s) {
+void launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s) {
   const int64_t nb = scan_blocks(in, n, partial, s);
   k_scan_down<true><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, partial, nb, e);
-  return nb > 1 ? 2 : 1;
 }
 
 void launch_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,

@@ -237,9 +237,8 @@ struct StepEnd {
   double* surf_time;
   unsigned long long* cyc;
 };
-// Scan of the new histogram (n > 0 cells) and end of the step; the number of
-// launches.
-int launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s);
+// Scan of the new histogram (n > 0 cells) and end of the step.
+void launch_scan_end(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, const StepEnd& e, cudaStream_t s);
 int64_t scan_partial_size(int64_t n);
 // An upload's particle counts (Mtot = M, Mcur = *kept) and first Delta t (from
 // dt_min, which is reset; *bad = 1 where an instance has neither a cell with
