@@ -23,6 +23,7 @@
 
 #include "../../include/sp.h"
 #include "sp_internal.h"
+#include "sp_schedule.h"
 
 using namespace sp;
 
@@ -1137,8 +1138,6 @@ sp_status sp_autotune(sp_ctx* c, int steps_per_trial, int* cap_out, int* warps_o
   if (!c || steps_per_trial < 1) return SP_ERR_ARG;
   sp_status s = ensure_ready(c);
   if (s != SP_OK) return s;
-  static const int caps[] = {128, 256, 384, 512, 768, 1024};
-  static const int warps[] = {2, 4, 8};
   const int cap0 = c->sched_cap, w0 = c->sched_warps;
   // collision-group time of steps_per_trial steps of the step graph (its
   // copy with timing events), after one untimed step (the batch partition
@@ -1161,22 +1160,9 @@ sp_status sp_autotune(sp_ctx* c, int steps_per_trial, int* cap_out, int* warps_o
   };
   struct Cand { int cap, warps; float t; };
   std::vector<Cand> cand;
-  // the fixed capacities, and for each block size the largest capacity at
-  // each residency level (blocks per SM from the occupancy calculator):
-  // more resident warps with slightly smaller batches can win (on the
-  // developed cylinder 864 x 2 at 6 blocks beat 1024 x 2 at 5 by 2 %)
-  std::vector<std::pair<int, int>> sched;
-  for (int wi : warps) {
-    for (int ci : caps) sched.push_back({ci, wi});
-    int last = -1;
-    for (int ci = kHugeCell; ci >= 128; ci -= 32) {
-      const int per = c->K->collide_blocks_per_sm(c->dim, wi, ci, c->n_inst == 1, c->subcells);
-      if (per != last && per > 0 &&
-          std::find(sched.begin(), sched.end(), std::make_pair(ci, wi)) == sched.end())
-        sched.push_back({ci, wi});
-      last = per;
-    }
-  }
+  const auto sched = schedule_candidates(
+      kHugeCell, [&](int cap, int w) { return c->K->collide_fits(w, cap); },
+      [&](int cap, int w) { return c->K->collide_blocks_per_sm(c->dim, w, cap, c->n_inst == 1, c->subcells); });
   for (const auto& sw : sched) {
     const int ci = sw.first, wi = sw.second;
     if (!apply_schedule(c, ci, wi)) continue;
