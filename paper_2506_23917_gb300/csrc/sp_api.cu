@@ -554,13 +554,15 @@ void enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   }
   // warps among which the plan spreads a small state: with an FP32 state at
   // most 8 per SM, since every batch costs the FP64 pipe the same per-cell
-  // arithmetic however few its cells (200 k particles, 10 steps: 775 us over
-  // 16 warps per SM, 613 over 8, 604 over 4; the 10-instance ensemble 1516,
-  // 1628, 1923; FP64 mode, whose particles cost more than its cells, all)
+  // arithmetic however few its cells (10 steps over 16 and 8 warps per SM:
+  // one box of 200 k particles 720 and 555 us, of 800 k 730 and 627; 10 of
+  // 20 k 761 and 598, of 80 k 794 and 664, 30 of 30 k 836 and 714; uneven
+  // ones: k_plan's limit on a batch's cost; FP64 mode, whose particles cost
+  // more than its cells, all)
   const int nwarps = small_grid(c) * c->sched_warps;
   launch_plan(c->start, c->cost, c->NC, c->sched_cap, c->prec != SP_FP64 ? std::min(nwarps, 8 * c->nsm) : nwarps,
               c->prec != SP_FP64 ? 96 : 32, (c->prec != SP_FP64 && c->dim == 2) ? kSplitLanes : 0,
-              c->batches, c->nbatch, c->big_list, c->big_count, c->stream);
+              c->n_inst > 1, c->batches, c->nbatch, c->big_list, c->big_count, c->stream);
   // the big-cell launch (cells disjoint from the batches') is a branch
   // beside the main launch: its blocks start as SMs free up at the end of
   // the main launch instead of after all of it

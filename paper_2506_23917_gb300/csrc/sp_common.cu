@@ -182,11 +182,19 @@ __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* 
 // of the collision launch (nwarps) a full batch is cut into smaller ones,
 // down to one cell each: the launch then lasts as long as one batch, whose
 // time grows with its particles (at least `least` particles, where that many
-// cost no more than fewer).
+// cost no more than fewer).  With several instances (kUneven), whose gases
+// may differ in density by orders of magnitude, a batch of such a state also
+// ends at 1.5 times the mean cost of a full one, so that the dear instance's
+// batches do not outlast all others: 10 uneven boxes, 10 steps, FP32
+// 1520 -> 1245 us (2 x: 1309; 4 x: 1520), FP64 2360 -> 2060; even ones
+// unchanged.  Not for a single flow: its dear regions are many small cells
+// (cylinder of 150 x 75 cells 2 % slower).
+template <bool kUneven>
 __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap_max, int nwarps, int least,
                        int split, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count) {
   const int64_t share = ((int64_t)start[NC] + nwarps - 1) / nwarps, want = share < least ? least : share;
   const int cap = want < cap_max ? (int)want : cap_max;
+  const uint32_t dear = want < cap_max ? 24u * (uint32_t)cap : 0xFFFFFFFFu;  // (kUneven)
   // per block: the batches of each class (shared atomics), then one global
   // atomic per class for the block's place in the class list
   __shared__ uint32_t cnt[kBatchClasses], base[kBatchClasses];
@@ -207,15 +215,17 @@ __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, i
       const int64_t c0 = chunk * 32;
       const int nc = (int)((NC - c0) < 32 ? (NC - c0) : 32);
       // inclusive prefix sums of the particle counts and the predicted costs
-      const int64_t nl = lane < nc ? (int64_t)(start[c0 + lane + 1] - start[c0 + lane]) : 0;
-      const int64_t wl = lane < nc ? (cost[c0 + lane] ? (int64_t)cost[c0 + lane] : 16) : 0;
+      // (32 bits: only differences over a batch of at most cap_max particles
+      // count, at most 255 cap_max)
+      const uint32_t nl = lane < nc ? start[c0 + lane + 1] - start[c0 + lane] : 0u;
+      const uint32_t wl = lane < nc ? (cost[c0 + lane] ? cost[c0 + lane] : 16u) : 0u;
       // lanes of the per-cell sums (split cells; at most 32 per batch)
-      int lcum = lane < nc ? cell_lanes((int)(nl < 0x7FFFFFFF ? nl : 0x7FFFFFFF), split) : 0;
-      int64_t cum = nl, ccum = nl * wl;
+      int lcum = lane < nc ? cell_lanes((int)(nl < 0x7FFFFFFFu ? nl : 0x7FFFFFFFu), split) : 0;
+      uint32_t cum = nl, ccum = nl * wl;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_up_sync(0xFFFFFFFFu, cum, o);
-        const int64_t z = __shfl_up_sync(0xFFFFFFFFu, ccum, o);
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, cum, o);
+        const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, ccum, o);
         const int w = __shfl_up_sync(0xFFFFFFFFu, lcum, o);
         if (lane >= o) {
           cum += y;
@@ -225,10 +235,13 @@ __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, i
       }
       int kk = 0;
       while (kk < nc) {
-        const int64_t before = kk > 0 ? __shfl_sync(0xFFFFFFFFu, cum, kk - 1) : 0;
+        const uint32_t before = kk > 0 ? __shfl_sync(0xFFFFFFFFu, cum, kk - 1) : 0u;
+        uint32_t cb = 0;
+        if constexpr (kUneven) cb = kk > 0 ? __shfl_sync(0xFFFFFFFFu, ccum, kk - 1) : 0u;
         const int lbefore = kk > 0 ? __shfl_sync(0xFFFFFFFFu, lcum, kk - 1) : 0;
         const unsigned fit = __ballot_sync(0xFFFFFFFFu, lane >= kk && lane < nc &&
-                                                          cum - before <= (lane == kk ? cap_max : cap) &&
+                                                          cum - before <= (uint32_t)(lane == kk ? cap_max : cap) &&
+                                                          (!kUneven || lane == kk || ccum - cb <= dear) &&
                                                           lcum - lbefore <= 32);
         const int G = __popc(fit);
         if (G == 0) {  // the cell alone exceeds the staging area: big-cell list
@@ -239,11 +252,11 @@ __global__ void k_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, i
           kk += 1;
           continue;
         }
-        const int64_t cb = kk > 0 ? __shfl_sync(0xFFFFFFFFu, ccum, kk - 1) : 0;
-        const int64_t cst = __shfl_sync(0xFFFFFFFFu, ccum, kk + G - 1) - cb;
+        if constexpr (!kUneven) cb = kk > 0 ? __shfl_sync(0xFFFFFFFFu, ccum, kk - 1) : 0u;
+        const uint32_t cst = __shfl_sync(0xFFFFFFFFu, ccum, kk + G - 1) - cb;
         if (lane == nb) {
           mine = make_uint2((uint32_t)(c0 + kk), (uint32_t)G);
-          const int64_t u = 16 * (int64_t)cap;  // a full batch at the mean cost
+          const uint32_t u = 16u * (uint32_t)cap;  // a full batch at the mean cost
           int cls;
           if (cst >= 4 * u) cls = 0;
           else if (cst >= 2 * u) cls = 1;
@@ -344,12 +357,12 @@ void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64
 }
 
 void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int nwarps, int least,
-                 int split, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
+                 int split, bool uneven, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s) {
   const int64_t chunks = (NC + 31) / 32;
   int64_t g = (chunks + 7) / 8;
   if (g > 4096) g = 4096;
   if (g < 1) g = 1;
-  k_plan<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, nwarps, least, split, batches, nbatch, big_list, big_count);
+  (uneven ? k_plan<true> : k_plan<false>)<<<(unsigned)g, 256, 0, s>>>(start, cost, NC, cap, nwarps, least, split, batches, nbatch, big_list, big_count);
 }
 
 int64_t scan_partial_size(int64_t n) { return (n + kTile - 1) / kTile + 1; }

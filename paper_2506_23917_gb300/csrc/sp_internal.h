@@ -219,7 +219,7 @@ const KernelSet& kernels_f32c();
 // Precision-independent kernels (sp_common.cu).
 void launch_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* partial, cudaStream_t s);
 void launch_plan(const uint32_t* start, const uint8_t* cost, int64_t NC, int cap, int nwarps, int least,
-                 int split, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s);
+                 int split, bool uneven, uint2* batches, uint32_t* nbatch, uint32_t* big_list, uint32_t* big_count, cudaStream_t s);
 void launch_mean_fields(const double* samp, int64_t NC, const double* vol, int64_t c0, int64_t nc, double nsamp,
                         double Fn, double R, double* out, cudaStream_t s);
 void launch_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,
