@@ -670,16 +670,12 @@ __device__ __forceinline__ bool move_particle(const InstParams& P, double* surf_
 // the walk as "outside".  Draws of wall event b: (step, sa, sb, purpose<<24
 // | subbase + 2b), as for the Cartesian walls.  Returns true when the
 // particle left the domain (or, locating, the point lies outside).
-// f0: the starting cell's face record (12 values) where the caller staged
-// it (shared memory), or null.
 template <class T>
 __device__ __forceinline__ bool mesh_walk(const InstParams& P, const T* mface, double* surf_all, int64_t& kl,
                                           T* x, T* v, T trem, uint32_t step, uint32_t purpose, uint32_t sa,
-                                          uint32_t sb, uint32_t subbase, unsigned long long* err, bool locate,
-                                          const T* f0 = nullptr) {
+                                          uint32_t sb, uint32_t subbase, unsigned long long* err, bool locate) {
   const Geo<T>& G = geo<T>(P);
   const int nr = P.n[0], nt = P.n[1];
-  const int64_t k0 = kl;
   int bounce = 0;
   for (int cross = 0;; ++cross) {
     if (cross >= kMaxCross) {
@@ -687,7 +683,7 @@ __device__ __forceinline__ bool mesh_walk(const InstParams& P, const T* mface, d
       atomicAdd(&err[kErrBounce], 1ull);
       return false;
     }
-    const T* f = (f0 != nullptr && kl == k0) ? f0 : mface + 12 * (P.cell_off + kl);
+    const T* f = mface + 12 * (P.cell_off + kl);
     if constexpr (sizeof(T) == 4) {
       // FP32 state: the flight that ends inside the cell (t_e >= trem on
       // every face it approaches, i.e. s_e >= trem (n_e . v)) is settled
@@ -1329,7 +1325,7 @@ __device__ __forceinline__ void record_conservation(const StepArgs& a, int64_t k
 // q_s).  FP64 mode: the oracle's expressions in its order.
 template <class A>
 struct CellMath {
-  A U[3], T, q[3], n, tau, dtc, ratio, dtG;
+  A U[3], T, q[3], n, tau, dtc, ratio;
   A RT, s2RT, Amax, omp;  // Shakhov sampling constants (shk)
   double Pres;            // resampling probability (shk)
   int64_t ncol;
@@ -1342,7 +1338,6 @@ struct CellMath {
     n = 0;
     tau = dtc = tinf<A>();
     ratio = 1;
-    dtG = 0;
     RT = s2RT = Amax = omp = 0;
     Pres = 0;
     ncol = 0;
@@ -1370,7 +1365,6 @@ __device__ __forceinline__ void cell_math_lean(const StepArgs& a, const InstPara
                                                int Ni, double m0, double m1, double m2, double mS2, double mS3x,
                                                double mS3y, double mS3z, double ivol_k, T smaxT, double dt_cur,
                                                uint32_t step, CellMath<double>& o) {
-  o.dtG = dt_cur;
   o.ratio = Pi.mode == 2 ? 0.0 : 1.0;  // cells without a split: the forced mode, else DSMC
   if (Ni <= 0) return;
   // 1/N, 1/(N-1), 1/(N-2) from the table of reciprocals (cells of the
@@ -1528,7 +1522,6 @@ __device__ __forceinline__ void cell_math(const StepArgs& a, const InstParams& P
   else if (Ni < 2 || !(Tt > (A)0) || dtct <= taut) o.ratio = 1;
   else o.ratio = cdiv(taut, dtct);
   const A dtG = (A)dt_cur;
-  o.dtG = dtG;
   if (Ni >= 2 && Tt > (A)0) {
     A dsmc, sbgk;
     if (Pi.mode == 1) { dsmc = dtG; sbgk = 0; }
@@ -2723,7 +2716,7 @@ struct __align__(16) HugeTab {
   A sum[8];              // the block's sums
   T wpm[kHugeWarps];     // prefix scans across warps (NTC passes)
   int wall[kHugeWarps];
-  T U[3], q[3], RT, s2RT, Amax, Pres, omp, dt, f, fl, Kh[3], Kl[3], smax;
+  T U[3], q[3], RT, s2RT, Amax, Pres, omp, f, fl, Kh[3], Kl[3], smax;
   A UA[3], TA;
   int ncol, nacc, nres, nar;
   double ratio;
@@ -2925,7 +2918,6 @@ __global__ void __launch_bounds__(kHugeThreads, 2) k_collide_huge(StepArgs a) {
       tb->Amax = (T)cm.Amax;
       tb->omp = (T)cm.omp;
       tb->Pres = cm.shk ? (T)cm.Pres : (T)0;
-      tb->dt = (T)cm.dtG;
       tb->smax = smaxT;
       tb->ncol = (int)cm.ncol;
       tb->nacc = 0;
