@@ -1,17 +1,19 @@
 // sp_api.cu -- host driver and C ABI of libsp (see include/sp.h).
 //
 // Per step the driver enqueues, on the context's stream:
-//   1. k_plan + k_collide (batches of cells per warp) and its
-//      big-cell launch (one warp per cell with a large staging area):
-//      gather through perm -> Step 3 moments -> Step 4
-//      DSMC / Shakhov / rescale -> Step 5 sums -> Step 2 free flight of the
-//      next interval, new key and histogram;
-//   2. reservoir injection at inflow faces (count, scan, write);
-//   3. exclusive scan of the histogram -> cell offsets of the new state, and
+//   1. k_plan + k_collide (batches of cells per warp), its big-cell launch
+//      (one warp per cell with a large staging area) and k_collide_huge (one
+//      block per cell): gather through perm -> Step 3 moments -> Step 4
+//      DSMC / Shakhov / rescale -> Step 5 sums -> velocities in cell order;
+//   2. k_flight: Step 2 free flight of the next interval, new key and
+//      histogram;
+//   3. beside both, reservoir injection at inflow faces (count, scan, write);
+//   4. exclusive scan of the histogram -> cell offsets of the new state, and
 //      bookkeeping (particle count, Delta t of the next step, step index);
-//   4. scatter of source indices into the new cell order (the histogram is
+//   5. scatter of source indices into the new cell order (the histogram is
 //      the cursor and ends at zero, ready for the next step), and in
-//      reproducible runs the source order inside each cell.
+//      reproducible runs the source order inside each cell (k_order_small,
+//      k_order_large).
 // The sequence is captured once per buffer parity as a CUDA graph and
 // replayed by sp_step().
 #include <algorithm>
@@ -530,7 +532,8 @@ bool apply_schedule(sp_ctx* c, int cap, int warps) {
 // capture into a step graph.  With ev != nullptr, event-record nodes
 // ev[0..4] bracket the four kernel groups (the plan and collision
 // launches; what is left of the injection branch when they end; the scan
-// and bookkeeping; the scatter), so that the host can time them.
+// and bookkeeping; the scatter and the in-cell order), so that the host can
+// time them.
 void enqueue_step(sp_ctx* c, int par, cudaEvent_t* ev = nullptr) {
   const StepArgs a = make_step_args(c, par);
   const auto rec = [&](int k) {

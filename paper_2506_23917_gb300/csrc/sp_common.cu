@@ -129,7 +129,7 @@ __global__ void k_scan_down(const uint32_t* in, uint32_t* out, int64_t n, const 
 // blocks run in about ascending order, and a cell fed by few of them often
 // arrives in source order.
 // The order inside a cell is arbitrary here; reproducible runs restore the
-// source order afterwards (k_order).
+// source order afterwards (k_order_small, k_order_large).
 constexpr int kScatterPer = 4;  // elements per thread, strided by the block size
 __global__ void k_scatter(const uint32_t* key, const uint32_t* start, uint32_t* count, uint32_t* perm,
                           const uint32_t* Mtot, int64_t cap) {

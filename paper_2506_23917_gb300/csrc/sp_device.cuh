@@ -1322,7 +1322,8 @@ __device__ __forceinline__ void record_conservation(const StepArgs& a, int64_t k
 // "Ncol_DSMC", fractional part by stochastic rounding or the carried
 // remainder), the resampling probability 1 - exp(-dt_SBGK / tau) (FP64) and
 // the Shakhov sampling constants (A_max at |C| = 5 sqrt(RT), C parallel to
-// q_s).  FP64 mode: the oracle's expressions in its order.
+// q_s).  FP64 mode: the oracle's expressions, operation for operation, on
+// the sums.
 template <class A>
 struct CellMath {
   A U[3], T, q[3], n, tau, dtc, ratio;
@@ -1770,7 +1771,7 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
     }
   }
   // ---- 1. source indices (in source order within each cell when the run is
-  // reproducible: k_order) and cell of each slot
+  // reproducible: k_order_small, k_order_large) and cell of each slot
 #pragma unroll 4
   for (int s = lane; s < M; s += 32) cp_async<4>(&sidx[s], &a.perm[p0 + s]);
   // the cell of slot sb + lane, for the 32 slots from sb (by the whole warp):
@@ -2380,7 +2381,8 @@ __device__ void process_batch(const StepArgs& a, int64_t k0, int G, CellTab<T, A
   A bsq[3] = {0, 0, 0};
   if (rcells) {
     if constexpr (!kMixed) {
-      // the U_p pass, then T_p about U_p (the oracle's order)
+      // the U_p pass, then T_p about U_p (as the oracle; inside a sum the
+      // order is cell_sums_acc's)
       A r1[3];
       cell_sums<Acc, 3>(lp, rown, offi, Ni, r1, [&](int s, int c, T* v, T* lo) {
         v[0] = svx[s];
@@ -2704,13 +2706,13 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock, sizeof(T) == 4 ? 2 : 1
 // cell in shared memory when it fits the launch's staging area and
 // otherwise in the cell's own output slots in global memory (velocities in
 // the B velocity arrays, source indices in the key array, clash tags in the
-// first B position array; the free flight overwrites all three last), so
+// first B position array; k_flight overwrites all three afterwards), so
 // no cell size is refused.  The steps are those of process_batch for one
 // cell: gather, two-pass moments, cell_math, the NTC loop
 // with exactly the one-by-one outcome (candidates of a round evaluated as
 // soon as their pair is final, decided against the prefix maximum of
 // sigma c), Shakhov resampling, the conservation rescale, Step 5 sums and
-// the free flight.
+// the velocities in cell order for k_flight.
 // ---------------------------------------------------------------------------
 template <class T, class A>
 struct __align__(16) HugeTab {
@@ -3754,12 +3756,12 @@ __device__ __forceinline__ double moment_sum(const double* sums, int64_t idx) {
   }
 }
 
-// FP64 state (kPair false): the oracle's arithmetic, operation for
-// operation (FP64 runs reproduce its Delta t and fields bit for bit).  FP32
-// state: the same quantities with the divisions taken as products of
-// reciprocals (1/k from the table, 1/V, 1/L) and the viscosity power as
-// tau = tau_k exp((omega - 1) ln T) / n: a few ulps from the quotient forms,
-// at a third of the FP64 instructions.
+// FP64 state (kPair false): the oracle's arithmetic, operation for operation,
+// on sums whose order is k_moment_sums' (so Delta t and fields agree with the
+// oracle's to the rounding of the sums).  FP32 state: the same quantities with
+// the divisions taken as products of reciprocals (1/k from the table, 1/V, 1/L)
+// and the viscosity power as tau = tau_k exp((omega - 1) ln T) / n: a few ulps
+// from the quotient forms, at a third of the FP64 instructions.
 template <bool kPair>
 __global__ void k_moment_cells(StepArgs a, int64_t c0, int64_t c1, const double* sums, double* out) {
   const int64_t nc = c1 - c0;

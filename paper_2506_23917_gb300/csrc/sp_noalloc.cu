@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kStaticThreads) k_static_scatter(const uint32_
 //   k_order_small  up to kSmallSeg: one warp per cell, up to 4 entries per lane;
 //   k_order_large  to kWarpSeg: one warp per cell, 8 to 32 entries per lane;
 //                  above: one block per cell (order_chunk, order_chunks).
-// Bound by instruction issue, about 2.4 warp-instructions per entry.
+// Bound by instruction issue (k_order_small: 4.5 warp-instructions per entry,
+// 76 % of the issue slots used).
 // k_order_small: 600 x 300 cylinder (6.6 M entries, 40 per cell) 35 us (48 by
 // the sorting network alone); sphere, 30 M entries in 1 M cells, 175 us (193).
 // k_order_large: jet, 4.5 M entries, most in cells of 500 to 2000, 66 us.
