@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kStaticThreads) k_static_scatter(const uint32_
 // 76 % of the issue slots used).
 // k_order_small: 600 x 300 cylinder (6.6 M entries, 40 per cell) 35 us (48 by
 // the sorting network alone); sphere, 30 M entries in 1 M cells, 175 us (193).
-// k_order_large: jet, 4.5 M entries, most in cells of 500 to 2000, 66 us.
+// k_order_large: jet, 5.9 M entries, most in cells of 500 to 2000, 46 us.
 // Restoring the order inside the collision kernel instead (12 resident warps
 // per SM, one shared-memory read per comparison) took 0.15, 0.38 and 0.38 ms
 // of those flows' steps.
